@@ -223,12 +223,14 @@ mka_status mka_cg_patch_targets(mka_system* sys, const int64_t* atoms, int64_t n
   const int max_cl = *std::max_element(sizes.begin(), sizes.end());
   if (max_cl > MKA_MAX_CLUSTER_ATOMS) return fail(MKA_ERR_CLUSTER_TOO_LARGE, "cluster larger than the cap");
   AtomsConfig cf{};
-  s = atoms_config(sys, 1, arith, max_cl, 256, 0, &cf);     // basis unused: smallest subspace
+  AtomsShape sh;                                             // basis unused: smallest subspace
+  sh.arith = arith;
+  sh.cg_only = 1;
+  s = atoms_config(sys, sh, max_cl, 256, 0, &cf);
   if (s) return s;
   cudaStream_t st = (cudaStream_t)stream;
-  const int64_t grid = std::min<int64_t>(n, cf.grid_max);
   char* buf = nullptr;
-  const size_t scratch_bytes = cf.slot_bytes * grid + 256;
+  const size_t scratch_bytes = (atoms_scratch_bytes(cf, n) + 255) / 256 * 256;
   const size_t extra = sizeof(int64_t) * n + sizeof(int32_t) * 8 * n + 256;
   MKA_CUDA_TRY(cudaMallocAsync(&buf, scratch_bytes + extra, st));
   int64_t* d_sel = reinterpret_cast<int64_t*>(buf + scratch_bytes);
@@ -236,7 +238,7 @@ mka_status mka_cg_patch_targets(mka_system* sys, const int64_t* atoms, int64_t n
   int32_t* d_iters = d_status + 4 * n;
   int* counter = reinterpret_cast<int*>(d_iters + 4 * n);
   cudaError_t e = cudaMemcpyAsync(d_sel, sel.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(int) * kAtomsCounters, st);
   if (e != cudaSuccess) {
     cudaFreeAsync(buf, st);
     return cuda_fail(e, "mka_cg_patch_targets");
@@ -252,7 +254,6 @@ mka_status mka_cg_patch_targets(mka_system* sys, const int64_t* atoms, int64_t n
   a.cg_iters = iters ? iters : d_iters;
   a.scratch = buf;
   a.counter = counter;
-  a.grid = (int)grid;
   a.patch = patch;
   a.cg_only = 1;
   a.cg_target = Y;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string>
 #include <vector>
@@ -98,7 +99,15 @@ struct AtomsConfig {
   int mcap = 0;            // 4 x largest cluster
   int lnnz_cap = 0;        // local block capacity
   int clcap = 0;           // cluster list capacity: the power of two at or above the largest cluster
+  int chains = 0;          // 1: the short-recurrence kernel runs first, the general one on what it left
+  int chains_grid = 0;     // its SMs x resident CTAs, dynamic shared memory and work slot
+  size_t chains_smem = 0;
+  size_t chains_slot = 0;
 };
+// Subspaces up to this size run the short-recurrence kernel (chains.cu).
+constexpr int kChainsMaxNu = 48;
+// Ints behind AtomsLaunchArgs::counter: queue positions of the two kernels and the count of atoms left over.
+constexpr int kAtomsCounters = 4;
 
 // Arguments of one launch of the per-atom kernel over a selection.
 struct AtomsLaunchArgs {
@@ -117,7 +126,8 @@ struct AtomsLaunchArgs {
   double* vp = nullptr;
   const int64_t* blk_off = nullptr;
   char* scratch = nullptr;         // grid x slot_bytes
-  int* counter = nullptr;          // zero in stream order before the launch
+  int* counter = nullptr;          // [kAtomsCounters], zero in stream order before the launch
+  int32_t* redo = nullptr;         // [n_sel] atoms the short-recurrence kernel leaves to the general one
   int grid = 0;
   const float* x0 = nullptr;       // learned CG start on the patch [4 n_sel][68], or NULL
   const int32_t* patch = nullptr;  // [n_sel][17]
@@ -166,8 +176,29 @@ mka_status mlp_forward_enqueue(const mka_mlp* net, const float* X, int64_t B, fl
                                float* H2, float* Y, cudaStream_t st);
 int64_t mlp_work_floats(int64_t B);   // floats of forward/backward work buffers for B rows
 
-mka_status atoms_config(const mka_system* sys, int nu, int arith, int max_cl, int threads, int ctas_per_sm,
+// What the per-atom kernels are configured for.
+struct AtomsShape {
+  int p = 1, q = 0;
+  int arith = MKA_FP64;
+  int mode_b = 0;          // reading B: the general kernel only
+  int cg_only = 0;         // the inner CG only
+  int general_only = 0;    // no leftover list at hand: the general kernel only
+};
+mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl, int threads, int ctas_per_sm,
                         AtomsConfig* out);
+// The short-recurrence kernel (chains.cu): adds its launch shape to a configuration (cf->chains stays 0 when its
+// working set does not fit), and its launch.
+mka_status chains_config(const mka_system* sys, int nu, int arith, int ctas_per_sm, AtomsConfig* cf);
+mka_status chains_launch(const mka_system* sys, int arith, const AtomsConfig& cf, const AtomsLaunchArgs& a,
+                         cudaStream_t st);
+// Bytes of work slots the kernels need for selections of up to n atoms.
+inline size_t atoms_scratch_bytes(const AtomsConfig& cf, int64_t n) {
+  const size_t g = cf.slot_bytes * (size_t)std::min<int64_t>(n, cf.grid_max);
+  const size_t c = cf.chains ? cf.chains_slot * (size_t)std::min<int64_t>(n, cf.chains_grid) : 0;
+  return std::max(g, c) + 256;
+}
+// Raises a kernel's dynamic shared memory limit to the device's; *most (may be NULL) gets it.
+mka_status allow_shared(const void* kernel, size_t* most);
 // The batched reduced problems of a selection the per-atom kernel has just processed.
 mka_status reduced_for(const mka_system* sys, const AtomsLaunchArgs& a, cudaStream_t st);
 mka_status atoms_launch(const mka_system* sys, int arith, const AtomsConfig& cf, const AtomsLaunchArgs& a,

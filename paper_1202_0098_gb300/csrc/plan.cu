@@ -127,9 +127,9 @@ mka_status plan_alloc(mka_plan* P) {
   MKA_CUDA_TRY(cudaMalloc(&r->d_status, sizeof(int32_t) * 4 * A));
   MKA_CUDA_TRY(cudaMalloc(&r->d_vp, sizeof(double) * max_blocks * 16 * nu));
   MKA_CUDA_TRY(cudaMalloc(&r->d_cv, kept_buffer_bytes(4 * A, (int)nu)));
-  MKA_CUDA_TRY(cudaMalloc(&P->scratch, P->cf.slot_bytes * (size_t)P->grid + 256));
+  MKA_CUDA_TRY(cudaMalloc(&P->scratch, atoms_scratch_bytes(P->cf, A)));
   MKA_CUDA_TRY(cudaMalloc(&P->red, red_buffer_bytes(4 * A, (int)nu)));
-  MKA_CUDA_TRY(cudaMalloc(&P->counter, 256));
+  MKA_CUDA_TRY(cudaMalloc(&P->counter, sizeof(int) * (kAtomsCounters + A)));
   MKA_CUDA_TRY(cudaMalloc(&P->order, sizeof(int32_t) * A));
   MKA_CUDA_TRY(cudaMalloc(&P->sizes, sizeof(int32_t) * A));
   MKA_CUDA_TRY(cudaMalloc(&P->bins, sizeof(int32_t) * kSizeBins));
@@ -156,7 +156,7 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   MKA_CUDA_TRY(cudaMemcpyAsync(r->d_sel, P->h_stage, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
   MKA_CUDA_TRY(cudaMemcpyAsync(r->d_blk_off, P->h_stage + P->max_atoms, sizeof(int64_t) * (n + 1),
                                cudaMemcpyHostToDevice, st));
-  MKA_CUDA_TRY(cudaMemsetAsync(P->counter, 0, sizeof(int), st));
+  MKA_CUDA_TRY(cudaMemsetAsync(P->counter, 0, sizeof(int) * kAtomsCounters, st));
   const int32_t* order = nullptr;
   if (P->tune.order_by_size) {
     mka_status s = launch_cluster_sizes(P->sys, r->d_sel, n, P->sizes, st);
@@ -200,11 +200,11 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   a.blk_off = r->d_blk_off;
   a.scratch = P->scratch;
   a.counter = P->counter;
+  a.redo = P->counter + kAtomsCounters;
   a.red = P->red;
   a.cv = r->d_cv;
   a.col0 = 0;
   a.mode_b = P->prm.subspace == MKA_SUBSPACE_B;
-  a.grid = (int)std::min<int64_t>(n, P->grid);
   MKA_CUDA_TRY(cudaEventRecordWithFlags(P->k0, st, cudaEventRecordExternal));
   mka_status s = atoms_launch(P->sys, P->prm.arith, P->cf, a, st);
   if (s) return s;
@@ -294,12 +294,17 @@ mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_p
     delete P;
     return fail(MKA_ERR_CLUSTER_TOO_LARGE, "a cluster of the system exceeds MKA_MAX_CLUSTER_ATOMS");
   }
-  s = atoms_config(sys, prm->p + prm->q, prm->arith, P->max_cl, t.threads, t.ctas_per_sm, &P->cf);
+  AtomsShape sh;
+  sh.p = prm->p;
+  sh.q = prm->q;
+  sh.arith = prm->arith;
+  sh.mode_b = prm->subspace == MKA_SUBSPACE_B;
+  s = atoms_config(sys, sh, P->max_cl, t.threads, t.ctas_per_sm, &P->cf);
   if (s) {
     delete P;
     return s;
   }
-  P->grid = (int)std::min<int64_t>(P->max_atoms, P->cf.grid_max);
+  P->grid = (int)std::min<int64_t>(P->max_atoms, P->cf.chains ? P->cf.chains_grid : P->cf.grid_max);
   s = plan_alloc(P);
   if (s) {
     mka_plan_destroy(P);
