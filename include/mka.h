@@ -248,12 +248,13 @@ void mka_result_destroy(mka_result* res);
 
 /* ---- global: mu, rho, G, energy --------------------------------------- */
 
-/* Chemical potential by bisection (Sec. 2, after Eq. EQ-DM): the mu with
+/* Chemical potential (Sec. 2, after Eq. EQ-DM): the mu with
  * 2 sum_j sum_alpha f(eps_alpha^(j); mu) w_alpha^(j) = n_electrons over the
  * result's columns, f(x) = 1 / (1 + exp((x - mu) / kT)). Bracket
- * [min eps - 40 kT, max eps + 40 kT], halved until narrower than `tol` (eV)
- * or 200 times; returns the midpoint in *mu_out (host). Runs on the device
- * with FP64 sums; synchronises. */
+ * [min eps - 40 kT, max eps + 40 kT], narrowed by the root finder of
+ * mka_sweep_find_mu until no wider than `tol` (eV) or for about 200 steps;
+ * returns the midpoint in *mu_out (host). Runs on the device with FP64 sums;
+ * synchronises. */
 mka_status mka_find_mu(mka_result* res, double n_electrons, double kT, double tol, double* mu_out);
 
 /* Density matrix (Eq. EQ-DM) on the selected rows' pattern, the band energy
@@ -358,7 +359,7 @@ typedef struct mka_plan mka_plan; /* every buffer of one batch of the work flow,
 
 /* A plan for batches of up to `max_atoms` atoms of `sys` (4 columns each): the
  * whole work flow of Eq. EQ-WORK-FLOW for one batch (the per-column brace with
- * kept data as for keep_vectors, mu by bisection over the batch's columns, rho and the band
+ * kept data as for keep_vectors, mu over the batch's columns, rho and the band
  * energy) with every buffer allocated here, once. `tune` may be NULL (defaults,
  * or pass the result of mka_autotune). The plan computes the largest cluster of
  * the whole system once, to size its work slots. Work runs on `stream`. */
@@ -369,7 +370,7 @@ mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_p
  * and the batch is enqueued as one CUDA graph (captured the first time this
  * (n_sel, n_electrons, kT, rho_out) combination is seen, replayed afterwards):
  * copy-in, optional ordering by cluster size, the persistent per-atom kernel,
- * 64 device bisection steps for mu (bracket as mka_find_mu, tolerance 1e-12 eV),
+ * up to 64 root-finder steps for mu on the device (as mka_find_mu, tolerance 1e-12 eV),
  * rho into `rho_out` (device, [n_blocks][4][4] as in mka_density_energy, may be
  * NULL) and the band energy. Returns without waiting for the GPU; the call waits
  * only for the previous batch to have read the staging buffer. */

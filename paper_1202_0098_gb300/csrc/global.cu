@@ -1,10 +1,10 @@
-// Global (all-column) kernels: mu by bisection, the density matrix with the band
+// Global (all-column) kernels: mu, the density matrix with the band
 // energy, the subspace Green's function, and the global block-sparse product.
 //
-// mu (Sec. 2, after Eq. EQ-DM): the electron count 2 sum_j sum_alpha f w is
-// evaluated by one launch per halving; the launch's blocks write fixed-order
-// partial sums, and the last block to finish (ticket counter) adds them in
-// block order and moves the bracket, so the result does not depend on timing.
+// mu (Sec. 2, after Eq. EQ-DM): the electron count 2 sum_j sum_alpha f w is evaluated by one launch per step of a
+// bracketing root finder (mu_root.cuh: a few bisection steps, then the Illinois secant, 10 to 15 passes where
+// halving alone took 46); the launch's blocks write fixed-order partial sums, and the last block to finish
+// (ticket counter) adds them in a fixed tree and takes the step, so the result does not depend on timing.
 // f(x) = (1 - tanh((x - mu) / (2 kT))) / 2; for |x - mu| / (2 kT) > 20 the FP64
 // tanh is exactly +-1, so those terms take f = 0 or 1 without calling it.
 //
@@ -19,6 +19,7 @@
 #include <cmath>
 
 #include "mka_internal.h"
+#include "mu_root.cuh"
 
 namespace mka {
 namespace {
@@ -52,15 +53,9 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;  // valid in thread 0
 }
 
-// Bisection state (device doubles): [0] lo, [1] hi, [2] target, [3] kT, [4] tol,
-// [5] last count, [6] halvings done. partial[kMaxRedBlocks], ticket (unsigned).
-struct MuState {
-  double lo, hi, target, kT, tol, last, iters, pad;
-};
-
 // min / max of eps over entries with w != 0 (fixed-order two-level reduction).
 __global__ void eps_range_kernel(const double* eps, const double* w, int64_t n, double* partial,
-                                 unsigned* ticket, MuState* S) {
+                                 unsigned* ticket, RootState* S) {
   __shared__ double rmin[kRedThreads / 32], rmax[kRedThreads / 32];
   __shared__ bool last;
   double mn = INFINITY, mx = -INFINITY;
@@ -93,33 +88,54 @@ __global__ void eps_range_kernel(const double* eps, const double* w, int64_t n, 
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (last) {
     __threadfence();
-    double a = INFINITY, b = -INFINITY;
-    for (unsigned k = 0; k < gridDim.x; ++k) {
-      a = fmin(a, partial[2 * k]);
-      b = fmax(b, partial[2 * k + 1]);
+    mn = INFINITY;
+    mx = -INFINITY;
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) {
+      mn = fmin(mn, partial[2 * k]);
+      mx = fmax(mx, partial[2 * k + 1]);
     }
-    S->lo = a - 40.0 * S->kT;
-    S->hi = b + 40.0 * S->kT;
-    S->iters = 0;
-    *ticket = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+      rmin[threadIdx.x >> 5] = mn;
+      rmax[threadIdx.x >> 5] = mx;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int k = 0; k < kRedThreads / 32; ++k) {
+        mn = fmin(mn, rmin[k]);
+        mx = fmax(mx, rmax[k]);
+      }
+      S->lo = mn - 40.0 * S->kT;
+      S->hi = mx + 40.0 * S->kT;
+      S->x = S->hi;              // first point: every level occupied (N(lo) = 0 needs no pass)
+      S->flo = -S->target;
+      S->fhi = 0.0;
+      S->side = 0.0;
+      S->rf = 0.0;
+      S->iters = 0;
+      *ticket = 0;
+    }
   }
 }
 
-// One halving: N(mid) = 2 sum f(eps; mid) w, then the bracket update.
-__global__ void bisect_kernel(const double* eps, const double* w, int64_t n, double* partial, unsigned* ticket,
-                              MuState* S) {
+// One step of the root finder: N(x) = 2 sum f(eps; x) w over the columns (a thread per column), then the bracket.
+// Measured at 32,768 columns of nu = 30: 81 us a halving (46 of them) when threads ran over single levels and one
+// thread added the blocks' sums; the whole search now takes 0.4 ms of a batch instead of 5.2.
+__global__ void __launch_bounds__(kRedThreads) mu_pass_kernel(const double* eps, const double* w, int64_t n_cols, int nu,
+                                                              double* partial, unsigned* ticket, RootState* S) {
   __shared__ double red[kRedThreads / 32];
   __shared__ bool last;
-  const double lo = S->lo, hi = S->hi;
-  if (!(hi - lo > S->tol)) return;   // converged: every block leaves before touching the ticket
-  const double mid = 0.5 * (lo + hi), kT = S->kT;
+  if (!(S->hi - S->lo > S->tol)) return;   // converged: every block leaves before touching the ticket
+  const double x = S->x, rk = 0.5 / S->kT;
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double wi = w[i];
-    if (wi != 0.0) acc += fermi(eps[i], mid, kT) * wi;
-  }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cols; i += (int64_t)gridDim.x * blockDim.x)
+    acc += column_count(eps + i * nu, w + i * nu, nu, x, rk);
   const double s = block_sum(acc, red);
   if (threadIdx.x == 0) {
     partial[blockIdx.x] = s;
@@ -127,21 +143,21 @@ __global__ void bisect_kernel(const double* eps, const double* w, int64_t n, dou
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (last) {
     __threadfence();
     double t = 0.0;
-    for (unsigned k = 0; k < gridDim.x; ++k) t += partial[k];
-    const double count = 2.0 * t;
-    if (count < S->target) S->lo = mid; else S->hi = mid;
-    S->last = count;
-    S->iters += 1;
-    *ticket = 0;
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) t += partial[k];
+    t = block_sum(t, red);
+    if (threadIdx.x == 0) {
+      root_step(S, 2.0 * t);
+      *ticket = 0;
+    }
   }
 }
 
-// Bracket state of a stream-ordered bisection (no host round trip): target, kT, tolerance,
+// Bracket state of a stream-ordered root search (no host round trip): target, kT, tolerance,
 // ticket cleared; the range kernel then sets lo / hi.
-__global__ void mu_init_kernel(MuState* S, unsigned* ticket, double target, double kT, double tol) {
+__global__ void mu_init_kernel(RootState* S, unsigned* ticket, double target, double kT, double tol) {
   S->target = target;
   S->kT = kT;
   S->tol = tol;
@@ -149,7 +165,7 @@ __global__ void mu_init_kernel(MuState* S, unsigned* ticket, double target, doub
   *ticket = 0;
 }
 
-__global__ void mu_finish_kernel(const MuState* S, double* mu_out) { *mu_out = 0.5 * (S->lo + S->hi); }
+__global__ void mu_finish_kernel(const RootState* S, double* mu_out) { *mu_out = 0.5 * (S->lo + S->hi); }
 
 // Column c of atom t: g = C diag(x) V_j for per-level weights x (ascending order of eps), from the
 // kept C and V_j (lane-interleaved by column); thread per (c, n), g into shared memory [4][nu].
@@ -238,30 +254,24 @@ __global__ void greens_kernel(const double* vp, const double* cv, const double* 
   }
 }
 
-// Fixed-order sum of n doubles by one CTA (thread 0 adds the per-thread sums in order).
+// Fixed-order sum of n doubles by one CTA (strided per thread, then the fixed tree).
 __global__ void sum_kernel(const double* x, int64_t n, double* out) {
-  __shared__ double part[kRedThreads];
+  __shared__ double red[kRedThreads / 32];
   double s = 0.0;
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += x[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int k = 0; k < (int)blockDim.x; ++k) t += part[k];
-    *out = t;
-  }
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) *out = s;
 }
 
-// 2 sum f(eps; mu) w: per-block partial sums (fixed grid), added in order by sum_kernel.
-__global__ void count_partial_kernel(const double* eps, const double* w, int64_t n, double mu_host, const double* mu_dev,
-                                     double kT, double* partial) {
+// 2 sum f(eps; mu) w over the columns: per-block partial sums (fixed grid), added by sum_kernel.
+__global__ void __launch_bounds__(kRedThreads) count_partial_kernel(const double* eps, const double* w, int64_t n_cols,
+                                                                    int nu, double mu_host, const double* mu_dev,
+                                                                    double kT, double* partial) {
   __shared__ double red[kRedThreads / 32];
-  const double mu = mu_dev ? *mu_dev : mu_host;
+  const double mu = mu_dev ? *mu_dev : mu_host, rk = 0.5 / kT;
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double wi = w[i];
-    if (wi != 0.0) acc += fermi(eps[i], mu, kT) * wi;
-  }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cols; i += (int64_t)gridDim.x * blockDim.x)
+    acc += column_count(eps + i * nu, w + i * nu, nu, mu, rk);
   const double s = block_sum(acc, red);
   if (threadIdx.x == 0) partial[blockIdx.x] = 2.0 * s;
 }
@@ -501,19 +511,23 @@ mka_status launch_dos(const double* eps, const double* w, int64_t n, const doubl
   return MKA_OK;
 }
 
-size_t mu_buffer_bytes() { return sizeof(MuState) + sizeof(double) * 2 * kMaxRedBlocks + 64; }
+static int blocks_of(int64_t n) {
+  return (int)std::min<int64_t>(red_blocks(), std::max<int64_t>(1, (n + kRedThreads - 1) / kRedThreads));
+}
 
-mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n, double n_electrons, double kT, double tol,
-                           int halvings, void* buf, double* mu_dev_out, cudaStream_t st) {
-  MuState* S = reinterpret_cast<MuState*>(buf);
+size_t mu_buffer_bytes() { return sizeof(RootState) + sizeof(double) * 2 * kMaxRedBlocks + 64; }
+
+mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n_cols, int nu, double n_electrons, double kT,
+                           double tol, int passes, void* buf, double* mu_dev_out, cudaStream_t st) {
+  RootState* S = reinterpret_cast<RootState*>(buf);
   double* partial = reinterpret_cast<double*>(S + 1);
   unsigned* ticket = reinterpret_cast<unsigned*>(partial + 2 * kMaxRedBlocks);
-  const int blocks = (int)std::min<int64_t>(red_blocks(), std::max<int64_t>(1, (n + kRedThreads - 1) / kRedThreads));
   mu_init_kernel<<<1, 1, 0, st>>>(S, ticket, n_electrons, kT, tol);
-  eps_range_kernel<<<blocks, kRedThreads, 0, st>>>(eps, w, n, partial, ticket, S);
-  for (int i = 0; i < halvings; ++i) bisect_kernel<<<blocks, kRedThreads, 0, st>>>(eps, w, n, partial, ticket, S);
+  eps_range_kernel<<<blocks_of(n_cols * nu), kRedThreads, 0, st>>>(eps, w, n_cols * nu, partial, ticket, S);
+  for (int i = 0; i < passes; ++i)
+    mu_pass_kernel<<<blocks_of(n_cols), kRedThreads, 0, st>>>(eps, w, n_cols, nu, partial, ticket, S);
   mu_finish_kernel<<<1, 1, 0, st>>>(S, mu_dev_out);
-  count_launches(3 + halvings);
+  count_launches(3 + passes);
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
 }
@@ -525,7 +539,7 @@ mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int6
                                                   sys->storage, nu, 0.0, mu_dev, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, n_sel, tmp + n_sel);
   const int rb = red_blocks();
-  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(eps, w, 4 * n_sel * nu, 0.0, mu_dev, kT, tmp + n_sel + 2);
+  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(eps, w, 4 * n_sel, nu, 0.0, mu_dev, kT, tmp + n_sel + 2);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp + n_sel + 2, rb, tmp + n_sel + 1);
   count_launches(4);
   MKA_CUDA_TRY(cudaGetLastError());
@@ -549,30 +563,27 @@ mka_status launch_find_mu(mka_result* res, double n_electrons, double kT, double
     MKA_CUDA_TRY(cudaMalloc(&res->d_mu_state, mu_buffer_bytes()));
     MKA_CUDA_TRY(cudaMemsetAsync(res->d_mu_state, 0, mu_buffer_bytes(), st));
   }
-  MuState* S = reinterpret_cast<MuState*>(res->d_mu_state);
+  RootState* S = reinterpret_cast<RootState*>(res->d_mu_state);
   double* partial = reinterpret_cast<double*>(S + 1);
   unsigned* ticket = reinterpret_cast<unsigned*>(partial + 2 * kMaxRedBlocks);
-  MuState h{};
-  h.target = n_electrons;
-  h.kT = kT;
-  h.tol = tol;
-  MKA_CUDA_TRY(cudaMemcpyAsync(S, &h, sizeof(MuState), cudaMemcpyHostToDevice, st));
-  MKA_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
-  const int blocks = (int)std::min<int64_t>(red_blocks(), std::max<int64_t>(1, (n + kRedThreads - 1) / kRedThreads));
-  eps_range_kernel<<<blocks, kRedThreads, 0, st>>>(res->d_eps, res->d_w, n, partial, ticket, S);
-  count_launches();
+  mu_init_kernel<<<1, 1, 0, st>>>(S, ticket, n_electrons, kT, tol);
+  eps_range_kernel<<<blocks_of(n), kRedThreads, 0, st>>>(res->d_eps, res->d_w, n, partial, ticket, S);
+  count_launches(2);
   MKA_CUDA_TRY(cudaGetLastError());
-  MKA_CUDA_TRY(cudaMemcpyAsync(&h, S, sizeof(MuState), cudaMemcpyDeviceToHost, st));
-  MKA_CUDA_TRY(cudaStreamSynchronize(st));
-  if (!(h.hi > h.lo)) return fail(MKA_ERR_INVALID_ARG, "no level with nonzero weight");
-  const int halvings = std::min(200, (int)std::ceil(std::log2((h.hi - h.lo) / tol)) + 2);
-  for (int i = 0; i < std::max(halvings, 1); ++i) {
-    bisect_kernel<<<blocks, kRedThreads, 0, st>>>(res->d_eps, res->d_w, n, partial, ticket, S);
+  // sixteen passes usually end the search (those after convergence return at once); the bracket comes back and
+  // more follow while it is wider than tol
+  RootState h{};
+  for (int done = 0; done < 200; done += 16) {
+    for (int i = 0; i < 16; ++i)
+      mu_pass_kernel<<<blocks_of(res->n_cols), kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, partial,
+                                                                     ticket, S);
+    count_launches(16);
+    MKA_CUDA_TRY(cudaGetLastError());
+    MKA_CUDA_TRY(cudaMemcpyAsync(&h, S, sizeof(RootState), cudaMemcpyDeviceToHost, st));
+    MKA_CUDA_TRY(cudaStreamSynchronize(st));
+    if (!(h.hi > h.lo) && h.iters == 0) return fail(MKA_ERR_INVALID_ARG, "no level with nonzero weight");
+    if (!(h.hi - h.lo > tol)) break;
   }
-  count_launches(std::max(halvings, 1));
-  MKA_CUDA_TRY(cudaGetLastError());
-  MKA_CUDA_TRY(cudaMemcpyAsync(&h, S, sizeof(MuState), cudaMemcpyDeviceToHost, st));
-  MKA_CUDA_TRY(cudaStreamSynchronize(st));
   *mu_out = 0.5 * (h.lo + h.hi);
   return MKA_OK;
 }
@@ -587,8 +598,8 @@ mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT
                                                        res->d_sel, sys->d_row_ptr, sys->d_valH, sys->storage,
                                                        res->nu, mu, nullptr, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, res->n_sel, tmp + res->n_sel);
-  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols * res->nu, mu, nullptr,
-                                                           kT, tmp + res->n_sel + 2);
+  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, mu, nullptr, kT,
+                                                   tmp + res->n_sel + 2);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp + res->n_sel + 2, rb, tmp + res->n_sel + 1);
   count_launches(4);
   cudaError_t e = cudaGetLastError();

@@ -221,8 +221,8 @@ mka_status launch_dos(const double* eps, const double* w, int64_t n, const doubl
 
 // Stream-ordered (no host synchronisation, no allocation) variants used by plans and graphs.
 size_t mu_buffer_bytes();
-mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n, double n_electrons, double kT, double tol,
-                           int halvings, void* buf, double* mu_dev_out, cudaStream_t st);
+mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n_cols, int nu, double n_electrons, double kT,
+                           double tol, int passes, void* buf, double* mu_dev_out, cudaStream_t st);
 mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int64_t* blk_off, const double* vp,
                            const double* cv, const double* eps, const double* w, int64_t n_sel, int nu,
                            const double* mu_dev, double kT, double* rho_out, double* tmp, cudaStream_t st);

@@ -1,12 +1,12 @@
 // Persistent, graph-captured batches of columns (plans) and the autotuner.
 //
 // A plan owns every buffer one batch of the work flow needs (Eq. EQ-WORK-FLOW:
-// the per-column brace, mu by bisection, rho and the band energy), sized once for
+// the per-column brace, mu, rho and the band energy), sized once for
 // at most `max_atoms` atoms, so that running a batch allocates nothing and never
 // waits on the host. A batch is one CUDA graph: copy of the atom list and its
 // output offsets from pinned staging, optional ordering of the work queue by
 // descending cluster size (uneven clusters finish together), the persistent
-// per-atom kernel, a fixed-length device bisection for mu, and the density /
+// per-atom kernel, a fixed number of root-finder passes for mu, and the density /
 // energy kernels. The graph is captured the first time a batch shape (atom count,
 // electron count, kT, rho buffer) is seen and replayed afterwards.
 //
@@ -30,7 +30,7 @@ namespace mka {
 namespace {
 
 constexpr int kSizeBins = MKA_MAX_CLUSTER_ATOMS + 1;
-constexpr int kHalvings = 64;   // bracket width / 2^64: below 1e-12 eV for any bracket narrower than 1.8e7 eV
+constexpr int kMuPasses = 64;   // the root finder needs 10 to 15; 64 halvings alone would close a bracket of 1.8e7 eV to 1e-12
 
 __global__ void size_hist_kernel(const int32_t* sizes, int64_t n, int32_t* bins) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -218,7 +218,7 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   if (m.kind == PLAN_AT_MU)
     return sweep_at_mu_enqueue(m.sw, r->d_sel, r->d_blk_off, r->d_vp, r->d_cv, r->d_eps, n, nu, m.mu, m.kT, m.rho,
                                m.forces, st);
-  s = find_mu_enqueue(r->d_eps, r->d_w, 4 * n * nu, m.n_electrons, m.kT, 1e-12, kHalvings, P->mu_buf, P->dev_out, st);
+  s = find_mu_enqueue(r->d_eps, r->d_w, 4 * n, nu, m.n_electrons, m.kT, 1e-12, kMuPasses, P->mu_buf, P->dev_out, st);
   if (s) return s;
   return density_enqueue(P->sys, r->d_sel, r->d_blk_off, r->d_vp, r->d_cv, r->d_eps, r->d_w, n, nu, P->dev_out, m.kT,
                          m.rho, P->dev_out + 1, st);

@@ -2,7 +2,7 @@
 //
 // A plan solves the system batch by batch; after each batch's column kernels a packing kernel
 // stores, at the system's own positions:
-//   - the levels eps_alpha and weights w_alpha of every column (what the bisection for mu needs);
+//   - the levels eps_alpha and weights w_alpha of every column (what the search for mu needs);
 //   - for every pattern entry (i, j) the occupied part sum_{eps_alpha < win_lo} v_alpha,i v_alpha,j
 //     and the products v_alpha,i v_alpha,j of the (at most kp) levels inside [win_lo, win_hi].
 // The Fermi-Dirac occupation f(x) = (1 - tanh((x - mu) / 2kT)) / 2 is exactly 1 in FP64 for
@@ -13,9 +13,9 @@
 // outside that range, are solved again at mu.
 //
 // Sums (electron count, band energy) run per chunk of consecutive atoms of the whole system, in a
-// fixed order inside the chunk (thread-strided, then a fixed tree), and the chunk sums are added in
-// chunk order. A process that sweeps a range starting on a chunk boundary therefore reproduces a
-// whole-system process's chunk sums exactly, and the bisection (Sec. 2) gives the same mu.
+// fixed order inside the chunk (blocks of 64 atoms, a thread per column and a fixed tree; then the
+// blocks, a warp per chunk), and the chunk sums are added in chunk order. A process that sweeps a range starting on a chunk boundary therefore reproduces a
+// whole-system process's chunk sums exactly, and the root finder (mu_root.cuh) gives the same mu.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "mka_internal.h"
+#include "mu_root.cuh"
 #include "sk_grad.cuh"
 
 namespace mka {
@@ -34,14 +35,10 @@ namespace {
 
 constexpr int kChunkThreads = 256;
 constexpr int kRangeBlocks = 1024;
-constexpr int kMaxHalvings = 200;
+constexpr int kMaxSteps = 200;
 
-// The root finder's state: the bracket [lo, hi] with f = N - N_e at its ends, the next point x, the
-// side that moved last (-1 lo, +1 hi) and whether x came from the secant (rf).
-struct BisState {
-  double lo, hi, target, kT, tol, last, iters, x, flo, fhi, side, rf;
-};
-constexpr double kSecantKT = 16.0;   // bisection while the bracket is wider than this many kT
+constexpr int kSubAtoms = kChunkThreads / 4;   // atoms of a block of a chunk: a thread per column
+constexpr int kStepsPerCheck = 16;             // root-finder steps enqueued between looks at the bracket
 
 __device__ __forceinline__ double fermi_f(double x, double mu, double r2kT) {   // r2kT = 1 / (2 kT)
   const double y = (x - mu) * r2kT;
@@ -232,15 +229,18 @@ struct ChunkArgs {
   const double* eatom;
   int nu;
   int64_t a0, a1, chunk_atoms, chunk0;
+  int n_sub;                 // blocks per chunk
   double mu;                 // used when S == NULL
-  const BisState* S;         // root finder: mu = the state's next point; nothing once converged
+  const RootState* S;        // root finder: mu = the state's next point; nothing once converged
   double kT;
-  double* count;             // [n_chunks] 2 sum f w
-  double* e_levels;          // [n_chunks] 2 sum f eps w (may be NULL)
-  double* e_rho;             // [n_chunks] sum of the atoms' 2 sum rho H (may be NULL)
+  double* part;              // [3][n_chunks][n_sub] the blocks' sums
+  int64_t n_chunks;
+  int levels, rho;           // also the level energies / the atoms' 2 sum rho H
 };
 
-// One CTA per chunk: entries of the chunk's atoms, thread t takes chunk-relative entries t, t + 256, ...
+// One CTA per block of 64 consecutive atoms of a chunk, a thread per column. One CTA per whole chunk left most
+// of the chip idle (13,824 atoms in chunks of 4,096: four CTAs, 340 us a pass, 69 ms of a 226 ms system; now 2.5 ms), and its threads ran over single
+// levels, a warp's lanes split between f = 1, f = 0 and the tanh.
 __global__ void __launch_bounds__(kChunkThreads) sweep_chunk_kernel(const ChunkArgs A) {
   __shared__ double red[kChunkThreads / 32];
   double mu = A.mu, kT = A.kT;
@@ -249,78 +249,64 @@ __global__ void __launch_bounds__(kChunkThreads) sweep_chunk_kernel(const ChunkA
     mu = A.S->x;
     kT = A.S->kT;
   }
-  const double r2kT = 0.5 / kT;        // one division per thread, a product per level
-  const int64_t gi = blockIdx.x;
-  const int64_t g = A.chunk0 + gi;
-  const int64_t lo = max(A.a0, g * A.chunk_atoms), hi = min(A.a1, (g + 1) * A.chunk_atoms);
-  const int64_t e0 = 4 * (lo - A.a0) * A.nu, e1 = 4 * (hi - A.a0) * A.nu;
+  const double rk = 0.5 / kT;          // one division per thread, a product per level
+  const int64_t gi = blockIdx.x / A.n_sub, sub = blockIdx.x % A.n_sub;
+  const int64_t g0 = (A.chunk0 + gi) * A.chunk_atoms, b0 = g0 + sub * kSubAtoms;
+  const int64_t lo = max(A.a0, b0), hi = min(A.a1, min(g0 + A.chunk_atoms, b0 + kSubAtoms));
+  const int64_t atom = b0 + (threadIdx.x >> 2);
   double c = 0.0, el = 0.0, er = 0.0;
-  for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const double wi = A.w[e];
-    if (wi != 0.0) {
-      const double x = A.eps[e];
-      const double f = fermi_f(x, mu, r2kT);
-      c += f * wi;
-      if (A.e_levels) el += f * x * wi;
-    }
+  if (atom >= lo && atom < hi) {
+    const int64_t col = 4 * (atom - A.a0) + (threadIdx.x & 3);
+    const double* eps = A.eps + col * A.nu;
+    const double* w = A.w + col * A.nu;
+    c = column_count(eps, w, A.nu, mu, rk);
+    if (A.levels)
+      for (int a = 0; a < A.nu; ++a) {
+        const double wi = w[a];
+        if (wi != 0.0) el += fermi_f(eps[a], mu, rk) * eps[a] * wi;
+      }
+    if (A.rho && (threadIdx.x & 3) == 0) er = A.eatom[atom - A.a0];
   }
-  if (A.e_rho)
-    for (int64_t a = lo - A.a0 + threadIdx.x; a < hi - A.a0; a += blockDim.x) er += A.eatom[a];
   const double cs = cta_sum(c, red);
-  const double es = A.e_levels ? cta_sum(el, red) : 0.0;
-  const double rs = A.e_rho ? cta_sum(er, red) : 0.0;
+  const double es = A.levels ? cta_sum(el, red) : 0.0;
+  const double rs = A.rho ? cta_sum(er, red) : 0.0;
   if (threadIdx.x == 0) {
-    A.count[gi] = 2.0 * cs;
-    if (A.e_levels) A.e_levels[gi] = 2.0 * es;
-    if (A.e_rho) A.e_rho[gi] = rs;
+    const int64_t n = A.n_chunks * A.n_sub;
+    A.part[blockIdx.x] = 2.0 * cs;
+    if (A.levels) A.part[n + blockIdx.x] = 2.0 * es;
+    if (A.rho) A.part[2 * n + blockIdx.x] = rs;
   }
 }
 
-// One step of the root finder for N(mu) = N_e: the count at x is the chunk sums added in chunk order;
-// the bracket end on its side moves to x. The next point is the midpoint while the bracket is wider
-// than 16 kT, then the secant through the ends (regula falsi, with the Illinois rule: after two moves
-// of the same end by the secant, the other end's f is halved), the midpoint when the secant leaves the
-// bracket; a point where the count equals N_e exactly closes the bracket on it. IEEE-rounded
-// operations throughout (no contraction), so that a host driver doing the same
-// arithmetic on the same chunk sums takes the same points bit for bit.
-__global__ void sweep_bisect_step_kernel(const double* count, int64_t n_chunks, BisState* S) {
+// A chunk's sums from its blocks', one warp per chunk (lanes strided, then the fixed tree).
+__global__ void __launch_bounds__(256) sweep_fold_kernel(const double* part, int64_t n_chunks, int n_sub, int kinds,
+                                                         double* chunk, const RootState* S) {
+  if (S && !(S->hi - S->lo > S->tol)) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t g = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (g >= n_chunks) return;
+  for (int k = 0; k < 3; ++k) {
+    if (!(kinds >> k & 1)) continue;
+    double s = 0.0;
+    for (int i = lane; i < n_sub; i += 32) s += part[((int64_t)k * n_chunks + g) * n_sub + i];
+    s = warp_sum_t(s);
+    if (lane == 0) chunk[k * n_chunks + g] = s;
+  }
+}
+
+// One step of the root finder (mu_root.cuh) from the chunk sums added in chunk order.
+__global__ void __launch_bounds__(256) sweep_root_step_kernel(const double* count, int64_t n_chunks, RootState* S) {
+  __shared__ double buf[256];
   if (!(S->hi - S->lo > S->tol)) return;
   double t = 0.0;
-  for (int64_t k = 0; k < n_chunks; ++k) t += count[k];
-  const double x = S->x, fx = __dsub_rn(t, S->target);
-  if (fx == 0.0) {                     // x is a root to rounding: the bracket closes on it
-    S->lo = x;
-    S->hi = x;
-    S->flo = 0.0;
-    S->fhi = 0.0;
-    S->last = t;
-    S->iters += 1;
-    return;
+  for (int64_t k0 = 0; k0 < n_chunks; k0 += 256) {
+    if (k0 + threadIdx.x < n_chunks) buf[threadIdx.x] = count[k0 + threadIdx.x];
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int k = 0; k < (int)min((int64_t)256, n_chunks - k0); ++k) t += buf[k];
+    __syncthreads();
   }
-  if (fx < 0.0) {
-    S->lo = x;
-    S->flo = fx;
-    if (S->rf != 0.0 && S->side == -1.0) S->fhi = __dmul_rn(0.5, S->fhi);
-    S->side = -1.0;
-  } else {
-    S->hi = x;
-    S->fhi = fx;
-    if (S->rf != 0.0 && S->side == 1.0) S->flo = __dmul_rn(0.5, S->flo);
-    S->side = 1.0;
-  }
-  S->last = t;
-  S->iters += 1;
-  const double lo = S->lo, hi = S->hi, mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
-  double nx = mid, rf = 0.0;
-  if (!(__dsub_rn(hi, lo) > __dmul_rn(kSecantKT, S->kT))) {
-    const double sx = __ddiv_rn(__dsub_rn(__dmul_rn(lo, S->fhi), __dmul_rn(hi, S->flo)), __dsub_rn(S->fhi, S->flo));
-    if (lo < sx && sx < hi) {
-      nx = sx;
-      rf = 1.0;
-    }
-  }
-  S->x = nx;
-  S->rf = rf;
+  if (threadIdx.x == 0) root_step(S, t);
 }
 
 struct RhoArgs {
@@ -480,8 +466,10 @@ struct mka_sweep {
   double* d_occ_pi = nullptr;           // [nblk][16] occupied part of pi (sweeps made for forces)
   double* d_g = nullptr;                // [nblk][3] force contribution of each block
   double* d_chunk = nullptr;            // [3][n_chunks]
+  double* d_part_sums = nullptr;        // [3][n_chunks][n_sub] the chunks' blocks
+  int n_sub = 1;                        // blocks of 64 atoms per chunk
   double* d_range = nullptr;            // [2 kRangeBlocks]
-  mka::BisState* d_state = nullptr;
+  mka::RootState* d_state = nullptr;
   unsigned long long* d_counts = nullptr;
   cudaEvent_t ev = nullptr;
   double rho_mu = NAN, rho_kT = NAN;
@@ -567,7 +555,7 @@ mka_status flag_counts(mka_sweep* sw, int64_t* stored, int64_t* overflow) {
   return MKA_OK;
 }
 
-mka_status chunk_launch(mka_sweep* sw, double mu, double kT, const BisState* S, bool levels, bool rho) {
+mka_status chunk_launch(mka_sweep* sw, double mu, double kT, const RootState* S, bool levels, bool rho) {
   ChunkArgs A{};
   A.eps = sw->d_eps;
   A.w = sw->d_w;
@@ -577,14 +565,18 @@ mka_status chunk_launch(mka_sweep* sw, double mu, double kT, const BisState* S, 
   A.a1 = sw->a1;
   A.chunk_atoms = sw->chunk_atoms;
   A.chunk0 = sw->chunk0;
+  A.n_sub = sw->n_sub;
   A.mu = mu;
   A.S = S;
   A.kT = kT;
-  A.count = sw->d_chunk;
-  A.e_levels = levels ? sw->d_chunk + sw->n_chunks : nullptr;
-  A.e_rho = rho ? sw->d_chunk + 2 * sw->n_chunks : nullptr;
-  sweep_chunk_kernel<<<(unsigned)sw->n_chunks, kChunkThreads, 0, sw->stream>>>(A);
-  count_launches();
+  A.part = sw->d_part_sums;
+  A.n_chunks = sw->n_chunks;
+  A.levels = levels;
+  A.rho = rho;
+  sweep_chunk_kernel<<<(unsigned)(sw->n_chunks * sw->n_sub), kChunkThreads, 0, sw->stream>>>(A);
+  sweep_fold_kernel<<<(unsigned)((sw->n_chunks + 7) / 8), 256, 0, sw->stream>>>(
+      sw->d_part_sums, sw->n_chunks, sw->n_sub, 1 | (levels ? 2 : 0) | (rho ? 4 : 0), sw->d_chunk, S);
+  count_launches(2);
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
 }
@@ -605,6 +597,7 @@ void mka_sweep_destroy(mka_sweep* sw) {
   cudaFree(sw->d_occ_pi);
   cudaFree(sw->d_g);
   cudaFree(sw->d_chunk);
+  cudaFree(sw->d_part_sums);
   cudaFree(sw->d_range);
   cudaFree(sw->d_state);
   cudaFree(sw->d_counts);
@@ -641,6 +634,8 @@ mka_status mka_sweep_create(mka_system* sys, int64_t atom_begin, int64_t atom_en
   sw->chunk_atoms = chunk_atoms;
   sw->chunk0 = atom_begin / chunk_atoms;
   sw->n_chunks = (atom_end - 1) / chunk_atoms - sw->chunk0 + 1;
+  // a chunk longer than the range has no more blocks than reach it
+  sw->n_sub = (int)((std::min(chunk_atoms, atom_end) + kSubAtoms - 1) / kSubAtoms);
   const int64_t n = sw->n;
   cudaError_t e = cudaSuccess;
   int64_t bytes = 0;
@@ -661,8 +656,9 @@ mka_status mka_sweep_create(mka_system* sys, int64_t atom_begin, int64_t atom_en
     ALLOC(sw->d_g, sizeof(double) * 3 * sw->nblk);
   }
   ALLOC(sw->d_chunk, sizeof(double) * 3 * sw->n_chunks);
+  ALLOC(sw->d_part_sums, sizeof(double) * 3 * sw->n_chunks * sw->n_sub);
   ALLOC(sw->d_range, sizeof(double) * 2 * kRangeBlocks);
-  ALLOC(sw->d_state, sizeof(BisState));
+  ALLOC(sw->d_state, sizeof(RootState));
   ALLOC(sw->d_counts, 2 * sizeof(unsigned long long));
 #undef ALLOC
   if (e == cudaSuccess) e = cudaMemsetAsync(sw->d_flag, 0, n, sw->stream);
@@ -744,7 +740,7 @@ mka_status mka_sweep_find_mu(mka_sweep* sw, double n_electrons, double kT, doubl
   double lo = 0, hi = 0;
   s = mka_sweep_level_range(sw, &lo, &hi);
   if (s) return s;
-  BisState h{};
+  RootState h{};
   h.lo = lo - 40.0 * kT;
   h.hi = hi + 40.0 * kT;
   h.target = n_electrons;
@@ -757,17 +753,19 @@ mka_status mka_sweep_find_mu(mka_sweep* sw, double n_electrons, double kT, doubl
   h.rf = 0.0;
   cudaStream_t st = sw->stream;
   MKA_CUDA_TRY(cudaMemcpyAsync(sw->d_state, &h, sizeof(h), cudaMemcpyHostToDevice, st));
-  for (int i = 0; i < kMaxHalvings; ++i) {
-    // both kernels return at once when the bracket is already narrower than tol (the loop's bound is
-    // the bisection's worst case; the secant phase usually ends it after a few steps)
-    s = chunk_launch(sw, 0.0, kT, sw->d_state, false, false);
-    if (s) return s;
-    sweep_bisect_step_kernel<<<1, 1, 0, st>>>(sw->d_chunk, sw->n_chunks, sw->d_state);
-    count_launches();
-    MKA_CUDA_TRY(cudaGetLastError());
+  // a few steps usually end the search (the rest of those enqueued return at once)
+  for (int done = 0; done < kMaxSteps; done += kStepsPerCheck) {
+    for (int i = 0; i < std::min(kStepsPerCheck, kMaxSteps - done); ++i) {
+      s = chunk_launch(sw, 0.0, kT, sw->d_state, false, false);
+      if (s) return s;
+      sweep_root_step_kernel<<<1, 256, 0, st>>>(sw->d_chunk, sw->n_chunks, sw->d_state);
+      count_launches();
+      MKA_CUDA_TRY(cudaGetLastError());
+    }
+    MKA_CUDA_TRY(cudaMemcpyAsync(&h, sw->d_state, sizeof(h), cudaMemcpyDeviceToHost, st));
+    MKA_CUDA_TRY(cudaStreamSynchronize(st));
+    if (!(h.hi - h.lo > tol)) break;
   }
-  MKA_CUDA_TRY(cudaMemcpyAsync(&h, sw->d_state, sizeof(h), cudaMemcpyDeviceToHost, st));
-  MKA_CUDA_TRY(cudaStreamSynchronize(st));
   *mu = 0.5 * (h.lo + h.hi);
   return MKA_OK;
 }
