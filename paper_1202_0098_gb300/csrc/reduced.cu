@@ -55,6 +55,13 @@ struct Lane {
   __device__ double& Z(int i, int j) const { return b[(size_t)(2 * nu * nu + 2 * nu + i * nu + j) * 32]; }
 };
 
+// A lane's vector in shared memory, `step` entries apart.
+struct Strided {
+  double* p;
+  int step;
+  __device__ double& operator[](int k) const { return p[k * step]; }
+};
+
 // S_r = L L^T in the lower triangle of S (right-looking); rdiag[k] = 1 / L_kk.
 __device__ bool lane_cholesky(const Lane& M, int n, double* rdiag) {
   for (int k = 0; k < n; ++k) {
@@ -145,7 +152,8 @@ __device__ void lane_tridiag(const Lane& M, int n, double* d, double* e, double*
 // Eigenvalues of the tridiagonal (d, e) by the implicit-shift QL method (Bowdler, Martin,
 // Reinsch & Wilkinson, Numer. Math. 11, 1968), in place on d (e is destroyed); rotation
 // lengths from rsqrt(f^2 + g^2). False when an eigenvalue needs more than 60 sweeps.
-__device__ bool lane_tql_values(int n, double* d, double* e) {
+template <typename V>
+__device__ bool lane_tql_values(int n, V d, V e) {
   for (int l = 0; l < n; ++l) {
     for (int iter = 0;; ++iter) {
       int m = l;
@@ -190,11 +198,23 @@ __device__ bool lane_tql_values(int n, double* d, double* e) {
   return true;
 }
 
+// Ascending.
+template <typename V>
+__device__ void lane_sort(int n, V d) {
+  for (int a = 1; a < n; ++a) {
+    const double t = d[a];
+    int b = a - 1;
+    for (; b >= 0 && d[b] > t; --b) d[b + 1] = d[b];
+    d[b + 1] = t;
+  }
+}
+
 // Gaussian elimination with partial pivoting of the tridiagonal T - lam I (d, e): the multipliers and
 // row interchanges in (mlt, swp), U as reciprocal pivots r0 and the two superdiagonals (u1, u2); a
 // pivot that vanishes is replaced by `tiny`. One division per row.
-__device__ void lane_tri_factor(int n, const double* d, const double* e, double lam, double tiny, double* r0,
-                                double* u1, double* u2, double* mlt, int* swp) {
+template <typename V>
+__device__ void lane_tri_factor(int n, V d, V e, double lam, double tiny, double* r0, double* u1, double* u2,
+                                double* mlt, int* swp) {
   double a = d[0] - lam, bb = n > 1 ? e[0] : 0.0;   // the working row: a at column k, bb at k + 1
   for (int k = 0; k + 1 < n; ++k) {
     const double sub = e[k], dn = d[k + 1] - lam, sp = k + 2 < n ? e[k + 1] : 0.0;
@@ -341,12 +361,7 @@ __global__ void __launch_bounds__(128) reduced_kernel(const RedArgs A) {
     ok = lane_tql_values(n, p, v);
   }
   if (ok) {
-    for (int a = 1; a < n; ++a) {      // ascending
-      const double t = p[a];
-      int b = a - 1;
-      for (; b >= 0 && p[b] > t; --b) p[b + 1] = p[b];
-      p[b + 1] = t;
-    }
+    lane_sort(n, p);
     lane_tri_vectors(M, n, d, e, p, v, x4[0], x4[1], x4[2], x4[3], rank);
     lane_back_transform<NUCAP>(M, n, rdiag, tau, x4);
     for (int a = 0; a < n; ++a) {
@@ -395,7 +410,479 @@ __global__ void __launch_bounds__(128) reduced_kernel(const RedArgs A) {
   }
 }
 
+// ---- teams: several lanes per column ---------------------------------------------------------------
+// One lane per column needs 32 columns a warp, its matrices stream through L2 (22 KB a column and matrix), and a column
+// is one long serial chain: 6.9 ms for a single column of nu = 30, 15.9 ms for 32,768 (a third of the FP64 pipe),
+// 445 ms for 148 columns of nu = 100. Here TL lanes share a column and CPW = 32 / TL columns share a warp
+// (rows, or eigenvectors, strided over the lanes, so that the shrinking triangles keep the lanes busy and the square
+// roots and divisions still serve CPW columns), with L and the matrix packed in shared memory, element by element
+// [CPW]. Three launches, because the eigenvalues want the one-lane form: team_tridiag_kernel (Cholesky,
+// congruence, Householder), ql_kernel (QL values, a thread per column) and team_vectors_kernel (inverse iteration,
+// back-transform, outputs). The algorithm is the lane kernel's step by step; the sums' order differs.
+__device__ __forceinline__ int pk(int i, int j) { return i * (i + 1) / 2 + j; }
+
+// Between the kernels a column's d, e, tau, 1 / L_kk and eigenvalues sit in its scratch (4 nu + nu doubles).
+struct Scratch {
+  double* z;
+  int nu;
+  __device__ double& d(int k) const { return z[(size_t)k * 32]; }
+  __device__ double& e(int k) const { return z[(size_t)(nu + k) * 32]; }
+  __device__ double& tau(int k) const { return z[(size_t)(2 * nu + k) * 32]; }
+  __device__ double& rdiag(int k) const { return z[(size_t)(3 * nu + k) * 32]; }
+  __device__ double& lam(int k) const { return z[(size_t)(4 * nu + k) * 32]; }
+};
+__device__ __forceinline__ Scratch scratch_of(const Lane& M) { return Scratch{&M.Z(0, 0), M.nu}; }
+constexpr int kTeamMinNu = 5;   // the scratch has nu^2 doubles
+
+template <int CPW>
+__device__ __forceinline__ double team_sum(double v) {
+#pragma unroll
+  for (int o = 16; o >= CPW; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Doubles of shared memory per column: two packed triangles and three vectors.
+__host__ __device__ constexpr int team_doubles(int n) { return n * (n + 1) + 3 * n; }
+
+template <int TL, int NS>
+__global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
+  constexpr int CPW = 32 / TL;
+  extern __shared__ double sm[];
+  const int lane = threadIdx.x, c = lane % CPW, l = lane / CPW, nu = A.nu;
+  const int64_t col = (int64_t)blockIdx.x * CPW + c;
+  const bool real = col < A.n_cols;
+  const int64_t colr = real ? col : A.n_cols - 1;
+  const Lane M{A.blk + (size_t)(colr >> 5) * red_block_doubles(nu) * 32 + (colr & 31), nu};
+  const Scratch Z = scratch_of(M);
+  const int st_in = A.status[colr], n_in = A.nu_eff[colr];
+  const int n = real && st_in == RS_OK && n_in > 0 && n_in <= nu ? n_in : 0;
+  const int nm = __reduce_max_sync(0xffffffffu, n);
+  double* L = sm + c;                                     // packed lower triangles, [element][CPW]
+  double* H = L + (size_t)nm * (nm + 1) / 2 * CPW;
+  double* vv = H + (size_t)nm * (nm + 1) / 2 * CPW;
+  double* ww = vv + (size_t)nm * CPW;
+  double* rd = ww + (size_t)nm * CPW;
+  // S_r and H_r (upper triangle stored), padded to nm with the identity and zeros
+  for (int i = l; i < nm; i += TL)
+    for (int j = 0; j <= i; ++j) {
+      const bool in = i < n;
+      L[pk(i, j) * CPW] = in ? M.S(i, j) : (i == j ? 1.0 : 0.0);
+      H[pk(i, j) * CPW] = in ? M.H(j, i) : 0.0;
+    }
+  __syncwarp();
+  // Cholesky, a column at a time from the ones before
+  bool spd = true;
+  for (int k = 0; k < nm; ++k) {
+    double v[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      v[s] = i >= k && i < nm ? L[pk(i, k) * CPW] : 0.0;
+    }
+    for (int j = 0; j < k; ++j) {
+      const double lk = L[pk(k, j) * CPW];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (TL * (s + 1) > k && TL * s < nm) v[s] = fma(-(l + TL * s < nm ? L[pk(l + TL * s, j) * CPW] : 0.0), lk, v[s]);
+    }
+    double dk = 0.0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      if (s == k / TL) dk = v[s];
+    dk = __shfl_sync(0xffffffffu, dk, (k % TL) * CPW + c);
+    if (!(dk > 0.0)) {
+      spd = false;
+      dk = 1.0;
+    }
+    const double lkk = sqrt(dk), r = 1.0 / lkk;
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      if (i > k && i < nm) L[pk(i, k) * CPW] = v[s] * r;
+      if (i == k) {
+        L[pk(k, k) * CPW] = lkk;
+        rd[k * CPW] = r;
+      }
+    }
+    __syncwarp();
+  }
+  // X = L^{-1} H, upper triangle: row i of the packed lower triangle is column i of X, a lane's own
+  for (int j = 0; j < nm; ++j) {
+    double v[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      v[s] = i >= j && i < nm ? H[pk(i, j) * CPW] : 0.0;
+    }
+    for (int k = 0; k < j; ++k) {
+      const double lk = L[pk(j, k) * CPW];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (TL * (s + 1) > j && TL * s < nm) v[s] = fma(-(l + TL * s < nm ? H[pk(l + TL * s, k) * CPW] : 0.0), lk, v[s]);
+    }
+    const double r = rd[j * CPW];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      if (i >= j && i < nm) H[pk(i, j) * CPW] = v[s] * r;
+    }
+  }
+  __syncwarp();
+  // A = L^{-1} X^T, lower triangle, column by column: the known part A(j, k), k < j, then the substitution
+  for (int j = 0; j < nm; ++j) {
+    double v[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      v[s] = i >= j && i < nm ? H[pk(i, j) * CPW] : 0.0;
+    }
+    for (int k = 0; k < j; ++k) {
+      const double a = H[pk(j, k) * CPW];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (TL * (s + 1) > j && TL * s < nm) v[s] = fma(-(l + TL * s < nm ? L[pk(l + TL * s, k) * CPW] : 0.0), a, v[s]);
+    }
+    for (int k = j; k < nm; ++k) {
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (l + TL * s == k) H[pk(k, j) * CPW] = v[s] * rd[k * CPW];
+      __syncwarp();
+      const double a = H[pk(k, j) * CPW];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (TL * (s + 1) > k && TL * s < nm)
+          v[s] = fma(-(l + TL * s > k && l + TL * s < nm ? L[pk(l + TL * s, k) * CPW] : 0.0), a, v[s]);
+    }
+  }
+  // Householder reduction on the lower triangle; reflectors stay below the diagonal
+  for (int k = 0; k + 2 < nm; ++k) {
+    const bool on = k + 2 < n;                               // a smaller column of the warp is done: no reflector
+    double v[NS], s2 = 0.0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      v[s] = on && i > k && i < nm ? H[pk(i, k) * CPW] : 0.0;
+      s2 = fma(v[s], v[s], s2);
+    }
+    s2 = team_sum<CPW>(s2);
+    const double x0 = on ? H[pk(k + 1, k) * CPW] : 0.0;
+    const double nrm = sqrt(s2);
+    const double alpha = x0 >= 0.0 ? -nrm : nrm;
+    const double v0 = x0 - alpha;
+    const double vtv = s2 - x0 * x0 + v0 * v0;
+    const double tk = vtv > 0.0 ? 2.0 / vtv : 0.0;          // H_k = I - tk v v^T
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i = l + TL * s;
+      if (on && i == k + 1) {
+        v[s] = v0;
+        H[pk(k + 1, k) * CPW] = v0;
+      }
+      if (i < nm) vv[i * CPW] = v[s];
+    }
+    if (l == 0 && on) {
+      Z.d(k) = H[pk(k, k) * CPW];
+      Z.e(k) = alpha;
+      Z.tau(k) = tk;
+    }
+    __syncwarp();
+    double p[NS], pv = 0.0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) p[s] = 0.0;
+    for (int j = k + 1; j < nm; ++j) {                       // p = tk B v from B's lower triangle
+      const double vj = vv[j * CPW];
+      const int jr = pk(j, 0);
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (TL * (s + 1) > k + 1 && TL * s < nm) {
+          const int i = l + TL * s;
+          const int o = j <= i ? pk(i, j) : jr + i;
+          p[s] = fma(i > k && i < nm ? H[o * CPW] : 0.0, vj, p[s]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      p[s] *= tk;
+      pv = fma(p[s], v[s], pv);
+    }
+    pv = team_sum<CPW>(pv);
+    const double kc = 0.5 * tk * pv;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      p[s] = fma(-kc, v[s], p[s]);                           // w = p - kc v
+      if (l + TL * s < nm) ww[(l + TL * s) * CPW] = p[s];
+    }
+    __syncwarp();
+    for (int j = k + 1; j < nm; ++j) {                       // B -= v w^T + w v^T
+      const double vj = vv[j * CPW], wj = ww[j * CPW];
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        const int i = l + TL * s;
+        if (i >= j && i < nm) {
+          double* b = H + pk(i, j) * CPW;
+          *b = fma(-p[s], vj, fma(-v[s], wj, *b));
+        }
+      }
+    }
+    __syncwarp();
+  }
+  if (!real) return;
+  if (l == 0) {
+    if (n >= 2) {
+      Z.d(n - 2) = H[pk(n - 2, n - 2) * CPW];
+      Z.e(n - 2) = H[pk(n - 1, n - 2) * CPW];
+    }
+    if (n >= 1) {
+      Z.d(n - 1) = H[pk(n - 1, n - 1) * CPW];
+      Z.e(n - 1) = 0.0;
+    }
+    int stc = st_in;
+    if (n > 0 && !spd) stc = RS_NOT_SPD;
+    else if (stc == RS_OK && n == 0) stc = RS_NOT_SPD;
+    else if (stc == RS_OK && n < nu) stc = RS_BREAKDOWN;
+    A.status[col] = stc;
+    A.nu_eff[col] = spd ? n : 0;
+  }
+  for (int i = l; i < n; i += TL) {
+    for (int j = 0; j <= i; ++j) M.S(i, j) = L[pk(i, j) * CPW];
+    for (int j = 0; j < i; ++j) M.H(i, j) = H[pk(i, j) * CPW];
+    Z.rdiag(i) = rd[i * CPW];
+  }
+}
+
+// The eigenvalues, a thread per column (its d and e in shared memory), ascending. (FP32 values refined by Rayleigh
+// quotients were tried instead: 2.8 -> 0.3 ms here at 32,768 columns of nu = 30, but the iterations for close pairs,
+// which some lane of a warp always has, cost 5 ms in the vectors.)
+__global__ void __launch_bounds__(32) ql_kernel(const RedArgs A) {
+  extern __shared__ double sm[];
+  const int64_t col = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  if (col >= A.n_cols) return;
+  const int nu = A.nu, n = A.nu_eff[col];
+  if (n <= 0) return;
+  const Lane M{A.blk + (size_t)(col >> 5) * red_block_doubles(nu) * 32 + (col & 31), nu};
+  const Scratch Z = scratch_of(M);
+  const Strided d{sm + threadIdx.x, 32}, e{sm + (size_t)nu * 32 + threadIdx.x, 32};
+  for (int k = 0; k < n; ++k) {
+    d[k] = Z.d(k);
+    e[k] = Z.e(k);
+  }
+  if (!lane_tql_values(n, d, e)) {
+    A.status[col] = RS_NOT_SPD;
+    A.nu_eff[col] = 0;
+    return;
+  }
+  lane_sort(n, d);
+  for (int k = 0; k < n; ++k) Z.lam(k) = d[k];
+}
+
+// Eigenvectors and outputs. A lane takes the eigenvectors l, l + TL, ...: two inverse iterations with one factorisation;
+// the vectors of a cluster (neighbours closer than 1e-3 ||T||_1) are then made orthonormal in order by the whole team,
+// iterated once more and made orthonormal again. Q and L^{-T} are applied to up to four vectors at a time, and the column's
+// levels, weights, C and V_j written.
+template <int TL, int NS>
+__global__ void __launch_bounds__(32) team_vectors_kernel(const RedArgs A) {
+  constexpr int CPW = 32 / TL, NUCAP = TL * NS, R = NS < 4 ? NS : 4;
+  extern __shared__ double sm[];
+  const int lane = threadIdx.x, c = lane % CPW, l = lane / CPW, nu = A.nu;
+  const int64_t col = (int64_t)blockIdx.x * CPW + c;
+  const bool real = col < A.n_cols;
+  const int64_t colr = real ? col : A.n_cols - 1;
+  const Lane M{A.blk + (size_t)(colr >> 5) * red_block_doubles(nu) * 32 + (colr & 31), nu};
+  const Scratch Z = scratch_of(M);
+  const int n = real ? A.nu_eff[colr] : 0;
+  const int nm = __reduce_max_sync(0xffffffffu, n);
+  double* L = sm + c;
+  double* H = L + (size_t)nm * (nm + 1) / 2 * CPW;
+  double* d = H + (size_t)nm * (nm + 1) / 2 * CPW;
+  double* e = d + (size_t)nm * CPW;
+  double* lam = e + (size_t)nm * CPW;
+  double tn = 0.0;
+  for (int i = l; i < n; i += TL) {
+    for (int j = 0; j <= i; ++j) L[pk(i, j) * CPW] = M.S(i, j);
+    for (int j = 0; j < i; ++j) H[pk(i, j) * CPW] = M.H(i, j);
+    d[i * CPW] = Z.d(i);
+    e[i * CPW] = Z.e(i);
+    lam[i * CPW] = Z.lam(i);
+    H[pk(i, i) * CPW] = i + 2 < n ? Z.tau(i) : 0.0;          // tau on the reflectors' free diagonal
+  }
+  double rdl[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) rdl[s] = l + TL * s < n ? Z.rdiag(l + TL * s) : 0.0;
+  __syncwarp();                                              // the scratch is free: Z's columns go there
+  for (int k = 0; k < n; ++k)
+    tn = fmax(tn, fabs(d[k * CPW]) + fabs(e[k * CPW]) + (k > 0 ? fabs(e[(k - 1) * CPW]) : 0.0));
+  const double ortol = 1e-3 * tn, tiny = 2.2204460492503131e-16 * (tn > 0.0 ? tn : 1.0);
+  double x4[4][NUCAP], mlt[NUCAP];
+  int swp[NUCAP];
+  const Strided sd{d, CPW}, se{e, CPW};
+  double* x = x4[0];
+  for (int a = l; a < n; a += TL) {
+    for (int i = 0; i < n; ++i) {
+      const double t = 0.7548776662466927 * (i + 1) + 0.5698402909980532 * (a + 1);
+      x[i] = 0.5 + (t - floor(t));
+    }
+    lane_tri_factor(n, sd, se, lam[a * CPW], tiny, x4[1], x4[2], x4[3], mlt, swp);
+    for (int it = 0; it < 2; ++it) {
+      lane_tri_apply(n, x4[1], x4[2], x4[3], mlt, swp, x);
+      double s2 = 0.0;
+      for (int i = 0; i < n; ++i) s2 += x[i] * x[i];
+      const double sc = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
+      for (int i = 0; i < n; ++i) x[i] *= sc;
+    }
+    for (int i = 0; i < n; ++i) M.Z(i, a) = x[i];
+  }
+  __syncwarp();
+  for (int it = 0; it < 2; ++it) {
+    // clusters: orthonormal in order by the whole team, one more iteration, and again
+    if (it == 1) {
+      for (int a = l; a < n; a += TL) {
+        if (a == 0 || !(lam[a * CPW] - lam[(a - 1) * CPW] <= ortol)) continue;
+        for (int i = 0; i < n; ++i) x[i] = M.Z(i, a);
+        lane_tri_factor(n, sd, se, lam[a * CPW], tiny, x4[1], x4[2], x4[3], mlt, swp);
+        lane_tri_apply(n, x4[1], x4[2], x4[3], mlt, swp, x);
+        double s2 = 0.0;
+        for (int i = 0; i < n; ++i) s2 += x[i] * x[i];
+        const double sc = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
+        for (int i = 0; i < n; ++i) x[i] *= sc;
+        for (int i = 0; i < n; ++i) M.Z(i, a) = x[i];
+      }
+      __syncwarp();
+    }
+    int cs = 0;
+    bool any = false;
+    for (int a = 1; a < nm; ++a) {
+      if (a < n && lam[a * CPW] - lam[(a - 1) * CPW] > ortol) cs = a;
+      const int len = a < n ? a - cs : 0;
+      const int most = __reduce_max_sync(0xffffffffu, len);
+      if (most == 0) continue;
+      any = true;
+      for (int b = 0; b < most; ++b) {
+        const bool on = b < len;
+        double dot = 0.0;
+        if (on)
+          for (int i = l; i < n; i += TL) dot = fma(M.Z(i, cs + b), M.Z(i, a), dot);
+        dot = team_sum<CPW>(dot);
+        if (on)
+          for (int i = l; i < n; i += TL) M.Z(i, a) = fma(-dot, M.Z(i, cs + b), M.Z(i, a));
+      }
+      double s2 = 0.0;
+      if (len)
+        for (int i = l; i < n; i += TL) s2 = fma(M.Z(i, a), M.Z(i, a), s2);
+      s2 = team_sum<CPW>(s2);
+      const double sc = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
+      if (len)
+        for (int i = l; i < n; i += TL) M.Z(i, a) *= sc;
+      __syncwarp();
+    }
+    if (!any) break;
+  }
+  // 1 / L_kk over d, which the eigenvectors no longer need
+#pragma unroll
+  for (int s = 0; s < NS; ++s)
+    if (l + TL * s < n) d[(l + TL * s) * CPW] = rdl[s];
+  __syncwarp();
+  if (!real) return;
+  double* epsc = A.eps + col * nu;
+  double* wc = A.w + col * nu;
+  const int64_t ca = A.col0 + col;
+  double* out = A.cv ? A.cv + (size_t)(ca >> 5) * kept_block_doubles(nu) * 32 + (ca & 31) : nullptr;
+  for (int a0 = l; a0 < nu; a0 += R * TL) {
+    const int na = a0 < n ? min(R, (n - a0 + TL - 1) / TL) : 0;
+    for (int r = 0; r < na; ++r)
+      for (int i = 0; i < n; ++i) x4[r][i] = M.Z(i, a0 + TL * r);
+    for (int r = na; r < R; ++r)
+      for (int i = 0; i < n; ++i) x4[r][i] = 0.0;
+    if (na) {
+      for (int k = n - 3; k >= 0; --k) {                     // x <- (I - tau_k v_k v_k^T) x
+        const double tk = H[pk(k, k) * CPW];
+        double dot[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) dot[r] = 0.0;
+        for (int i = k + 1; i < n; ++i) {
+          const double vi = H[pk(i, k) * CPW];
+#pragma unroll
+          for (int r = 0; r < R; ++r) dot[r] = fma(vi, x4[r][i], dot[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) dot[r] *= tk;
+        for (int i = k + 1; i < n; ++i) {
+          const double vi = H[pk(i, k) * CPW];
+#pragma unroll
+          for (int r = 0; r < R; ++r) x4[r][i] = fma(-dot[r], vi, x4[r][i]);
+        }
+      }
+      for (int i = n - 1; i >= 0; --i) {                     // C = L^{-T} (Q Z)
+        double s[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) s[r] = x4[r][i];
+        for (int k = i + 1; k < n; ++k) {
+          const double lk = L[pk(k, i) * CPW];
+#pragma unroll
+          for (int r = 0; r < R; ++r) s[r] = fma(-lk, x4[r][k], s[r]);
+        }
+        const double ri = d[i * CPW];
+#pragma unroll
+        for (int r = 0; r < R; ++r) x4[r][i] = s[r] * ri;
+      }
+    }
+    double vj[R], svj[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) vj[r] = svj[r] = 0.0;
+    for (int k = 0; k < n; ++k) {
+      const double u = M.UJ(k), su = M.SUJ(k);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        vj[r] = fma(u, x4[r][k], vj[r]);
+        svj[r] = fma(su, x4[r][k], svj[r]);
+      }
+    }
+    for (int r = 0; r < R; ++r) {
+      const int a = a0 + TL * r;
+      if (a >= nu) break;
+      const bool in = r < na;
+      epsc[a] = in ? lam[a * CPW] : 0.0;
+      wc[a] = in ? vj[r] * svj[r] : 0.0;
+      if (out) {
+        for (int i = 0; i < nu; ++i) out[(size_t)(i * nu + a) * 32] = in && i < n ? x4[r][i] : 0.0;
+        out[(size_t)(nu * nu + a) * 32] = in ? vj[r] : 0.0;
+      }
+    }
+  }
+}
+
+// TL1 lanes a column in the first kernel, TL2 in the last; nu <= TL NS.
+template <int TL1, int NS1, int TL2, int NS2>
+mka_status team_launch(const RedArgs& A, cudaStream_t st) {
+  constexpr int C1 = 32 / TL1, C2 = 32 / TL2;
+  auto k1 = team_tridiag_kernel<TL1, NS1>;
+  auto k2 = team_vectors_kernel<TL2, NS2>;
+  mka_status s = allow_shared(reinterpret_cast<const void*>(k1), nullptr);
+  if (!s) s = allow_shared(reinterpret_cast<const void*>(ql_kernel), nullptr);
+  if (!s) s = allow_shared(reinterpret_cast<const void*>(k2), nullptr);
+  if (s) return s;
+  const size_t smem = sizeof(double) * team_doubles(A.nu);
+  k1<<<(unsigned)((A.n_cols + C1 - 1) / C1), 32, smem * C1, st>>>(A);
+  ql_kernel<<<(unsigned)((A.n_cols + 31) / 32), 32, sizeof(double) * 2 * A.nu * 32, st>>>(A);
+  k2<<<(unsigned)((A.n_cols + C2 - 1) / C2), 32, smem * C2, st>>>(A);
+  count_launches(3);
+  MKA_CUDA_TRY(cudaGetLastError());
+  return MKA_OK;
+}
+
 }  // namespace
+
+// Which form (milliseconds measured at nu = 30 / 40; lane: one lane per column):
+//   up to 2,048 columns a whole warp takes a column, the chip is not full (2,048: 2.8 against 9.3);
+//   then teams: 11,996 columns 6.4 against 10.8, 16,384 7.1 against 10.8, 32,768 14.3 against 15.9 (nu = 30);
+//   10,004 columns 15 against 23.9 (nu = 40);
+//   one lane per column once there are enough of them to fill the chip that way, it has no idle lanes (524,288
+//   columns of nu = 30: 158, 0.30 us a column against the teams' 0.44): from about 40,000 columns up to nu = 32, and
+//   16,000 up to nu = 64, where a lane's rate is 0.7 us and a team's 1.5;
+//   nu up to 160 (the packed triangles fit in shared memory): a warp per column at any count (148 columns of nu = 100:
+//   52 against 445); below nu = 5 the scratch between the three kernels does not fit.
+constexpr int64_t kFewColumns = 2048, kManyColumns32 = 40960, kManyColumns64 = 16384;
 
 mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
                           double* w, double* cv, int64_t col0, cudaStream_t st) {
@@ -410,6 +897,16 @@ mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, 
   A.w = w;
   A.cv = cv;
   A.col0 = col0;
+  if (nu >= kTeamMinNu && nu <= 160) {
+    if (nu > 64) return team_launch<32, 5, 32, 5>(A, st);
+    if (nu > 32) {
+      if (n_cols <= kFewColumns) return team_launch<32, 2, 32, 2>(A, st);
+      if (n_cols <= kManyColumns64) return team_launch<16, 4, 32, 2>(A, st);
+    } else {
+      if (n_cols <= kFewColumns) return team_launch<32, 1, 32, 1>(A, st);
+      if (n_cols <= kManyColumns32) return team_launch<8, 4, 16, 2>(A, st);
+    }
+  }
   const int threads = 128;
   const unsigned blocks = (unsigned)((n_cols + threads - 1) / threads);
   if (nu <= kTinyNu) reduced_kernel<kTinyNu><<<blocks, threads, 0, st>>>(A);
