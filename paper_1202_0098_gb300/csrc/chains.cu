@@ -17,7 +17,7 @@
 // W^T H W and W^T S W are summed at the end from the stored W, H W, S W, so lost orthogonality costs no
 // accuracy either, as long as W stays well conditioned. It is watched through q_1 = e_j: |(w_n)_j| is
 // the overlap of w_n with q_1. An atom goes to the general kernel (its index into `redo`) when that
-// exceeds 1e-4, when a vector keeps less than 1e-6 of its norm, when s_j keeps less than 1e-7 (unless all
+// exceeds 1e-3, when a vector keeps less than 1e-6 of its norm, when s_j keeps less than 1e-7 (unless all
 // four columns keep less than 1e-12: then s_j is in K_p, as for S = I, and the first chain simply
 // continues), when an inner CG failed, or when its cluster is small against the subspace (m < 6 nu:
 // there the recurrences lose orthogonality within 30 to 40 steps).
@@ -616,7 +616,7 @@ __device__ __forceinline__ void chain_scalars(double beta, double qv, double zv,
   from_double(-zv, sc[20 + c]);
 }
 
-constexpr double kOverlapMax = 1e-4;           // |w_n . e_j| beyond which an atom goes to the general kernel
+constexpr double kOverlapMax = 1e-3;           // |w_n . e_j| beyond which an atom goes to the general kernel
 
 // Beyond this the FP32 form takes H_r from a Gram matrix too, instead of from the recurrence coefficients (whose
 // error is about ||H|| times the lost orthogonality, up to a few hundred times the overlap with q_1).

@@ -1165,7 +1165,9 @@ mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_para
   if (s) return s;
   // atoms per chunk: the reduced-problem buffer of a chunk stays within 2 GiB
   const size_t per_atom = red_buffer_bytes(32, nu) / 8;
-  const int64_t chunk = std::max<int64_t>(8, std::min<int64_t>(res->n_sel, ((size_t)2 << 30) / per_atom) & ~(int64_t)7);
+  // (a multiple of 8 atoms, 32 columns, where another chunk follows; 37 atoms in chunks of 32 and 5 took twice the time)
+  const int64_t most = std::max<int64_t>(8, (int64_t)(((size_t)2 << 30) / per_atom) & ~(int64_t)7);
+  const int64_t chunk = std::min(res->n_sel, most);
   const int64_t cmax = std::min(res->n_sel, chunk);
   char* scratch = nullptr;
   int* counter = nullptr;
