@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(128) reduced_kernel(const RedArgs A) {
 // (rows, or eigenvectors, strided over the lanes, so that the shrinking triangles keep the lanes busy and the square
 // roots and divisions still serve CPW columns), with L and the matrix packed in shared memory, element by element
 // [CPW]. Three launches, because the eigenvalues want the one-lane form: team_tridiag_kernel (Cholesky,
-// congruence, Householder), ql_kernel (QL values, a thread per column) and team_vectors_kernel (inverse iteration,
+// congruence, Householder), ql_kernel (QL values, a thread per column; bisect_kernel for few) and team_vectors_kernel (inverse iteration,
 // back-transform, outputs). The algorithm is the lane kernel's step by step; the sums' order differs.
 __device__ __forceinline__ int pk(int i, int j) { return i * (i + 1) / 2 + j; }
 
@@ -677,6 +677,78 @@ __global__ void __launch_bounds__(32) ql_kernel(const RedArgs A) {
   for (int k = 0; k < n; ++k) Z.lam(k) = d[k];
 }
 
+// The eigenvalues of few columns, a thread per eigenvalue: bisection on the sign changes of the leading principal minors
+// of T - x I (Givens), p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2}. T is scaled by a power of two to |T| <= 1, so they
+// grow by at most 2.5 a row; a pair below 2^-333 is scaled up again, looked at every 8 rows; a zero counts as a distance
+// of 2^-60, far below the rounding of d_i. QL is one serial chain a column and an FP64 instruction holds a warp's scheduler for 64 cycles: 1.3 ms
+// at nu = 30 and 15 ms at nu = 100, whatever the number of columns; four FP64 operations a row and step make this
+// the shorter way up to kFewColumns, and the longer one beyond (six times the operations).
+__global__ void __launch_bounds__(32) bisect_kernel(const RedArgs A) {
+  extern __shared__ double sm[];
+  const int lane = threadIdx.x, nu = A.nu, groups = (nu + 31) / 32;
+  const int64_t col = blockIdx.x / groups;
+  const int a = (int)(blockIdx.x % groups) * 32 + lane, n = A.nu_eff[col];
+  if (n <= 0) return;
+  const Lane M{A.blk + (size_t)(col >> 5) * red_block_doubles(nu) * 32 + (col & 31), nu};
+  const Scratch Z = scratch_of(M);
+  double *d = sm, *e2 = sm + n;
+  double lo = INFINITY, hi = -INFINITY, big = 0.0;
+  bool finite = true;
+  for (int k = lane; k < n; k += 32) {
+    const double dk = Z.d(k), r = (k + 1 < n ? fabs(Z.e(k)) : 0.0) + (k > 0 ? fabs(Z.e(k - 1)) : 0.0);
+    finite &= fabs(dk) + r < INFINITY;
+    lo = fmin(lo, dk - r);
+    hi = fmax(hi, dk + r);
+    big = fmax(big, fabs(dk) + r);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+  }
+  if (!__all_sync(0xffffffffu, finite)) {                   // as a QL that does not converge
+    if (a == 0) {
+      A.status[col] = RS_NOT_SPD;
+      A.nu_eff[col] = 0;
+    }
+    return;
+  }
+  const int ex = big > 0.0 ? ilogb(big) + 1 : 0;
+  for (int k = lane; k < n; k += 32) {
+    const double ek = k + 1 < n ? ldexp(Z.e(k), -ex) : 0.0;
+    d[k] = ldexp(Z.d(k), -ex);
+    e2[k] = ek * ek;
+  }
+  __syncwarp();
+  lo = ldexp(lo, -ex) - 1e-15;
+  hi = ldexp(hi, -ex) + 1e-15;
+  for (int it = 0; it < 64 && hi - lo > 1e-16; ++it) {
+    const double x = 0.5 * (lo + hi);
+    if (!(lo < x && x < hi)) break;
+    double p0 = 1.0, p1 = d[0] - x;
+    if (p1 == 0.0) p1 = 0x1p-60;
+    int below = p1 < 0.0;
+    for (int i0 = 1; i0 < n; i0 += 8) {
+      if (max(__double2hiint(p0) & 0x7fffffff, __double2hiint(p1) & 0x7fffffff) < (1023 - 333) << 20) {
+        p0 *= 0x1p333;
+        p1 *= 0x1p333;
+      }
+      const int i1 = min(i0 + 8, n);
+      for (int i = i0; i < i1; ++i) {
+        double p = fma(d[i] - x, p1, -e2[i - 1] * p0);
+        if (p == 0.0) p = p1 * 0x1p-60;
+        below += (__double2hiint(p) ^ __double2hiint(p1)) < 0;
+        p0 = p1;
+        p1 = p;
+      }
+    }
+    if (below > a) hi = x;
+    else lo = x;
+  }
+  if (a < n) Z.lam(a) = ldexp(0.5 * (lo + hi), ex);
+}
+
 // Eigenvectors and outputs. A lane takes the eigenvectors l, l + TL, ...: two inverse iterations with one factorisation;
 // the vectors of a cluster (neighbours closer than 1e-3 ||T||_1) are then made orthonormal in order by the whole team,
 // iterated once more and made orthonormal again. Q and L^{-T} are applied to up to four vectors at a time, and the column's
@@ -852,27 +924,6 @@ __global__ void __launch_bounds__(32) team_vectors_kernel(const RedArgs A) {
   }
 }
 
-// TL1 lanes a column in the first kernel, TL2 in the last; nu <= TL NS.
-template <int TL1, int NS1, int TL2, int NS2>
-mka_status team_launch(const RedArgs& A, cudaStream_t st) {
-  constexpr int C1 = 32 / TL1, C2 = 32 / TL2;
-  auto k1 = team_tridiag_kernel<TL1, NS1>;
-  auto k2 = team_vectors_kernel<TL2, NS2>;
-  mka_status s = allow_shared(reinterpret_cast<const void*>(k1), nullptr);
-  if (!s) s = allow_shared(reinterpret_cast<const void*>(ql_kernel), nullptr);
-  if (!s) s = allow_shared(reinterpret_cast<const void*>(k2), nullptr);
-  if (s) return s;
-  const size_t smem = sizeof(double) * team_doubles(A.nu);
-  k1<<<(unsigned)((A.n_cols + C1 - 1) / C1), 32, smem * C1, st>>>(A);
-  ql_kernel<<<(unsigned)((A.n_cols + 31) / 32), 32, sizeof(double) * 2 * A.nu * 32, st>>>(A);
-  k2<<<(unsigned)((A.n_cols + C2 - 1) / C2), 32, smem * C2, st>>>(A);
-  count_launches(3);
-  MKA_CUDA_TRY(cudaGetLastError());
-  return MKA_OK;
-}
-
-}  // namespace
-
 // Which form (milliseconds measured at nu = 30 / 40; lane: one lane per column):
 //   up to 2,048 columns a whole warp takes a column, the chip is not full (2,048: 2.8 against 9.3);
 //   then teams: 11,996 columns 6.4 against 10.8, 16,384 7.1 against 10.8, 32,768 14.3 against 15.9 (nu = 30);
@@ -883,6 +934,31 @@ mka_status team_launch(const RedArgs& A, cudaStream_t st) {
 //   nu up to 160 (the packed triangles fit in shared memory): a warp per column at any count (148 columns of nu = 100:
 //   52 against 445); below nu = 5 the scratch between the three kernels does not fit.
 constexpr int64_t kFewColumns = 2048, kManyColumns32 = 40960, kManyColumns64 = 16384;
+
+// TL1 lanes a column in the first kernel, TL2 in the last; nu <= TL NS.
+template <int TL1, int NS1, int TL2, int NS2>
+mka_status team_launch(const RedArgs& A, cudaStream_t st) {
+  constexpr int C1 = 32 / TL1, C2 = 32 / TL2;
+  auto k1 = team_tridiag_kernel<TL1, NS1>;
+  auto k2 = team_vectors_kernel<TL2, NS2>;
+  mka_status s = allow_shared(reinterpret_cast<const void*>(k1), nullptr);
+  if (!s) s = allow_shared(reinterpret_cast<const void*>(ql_kernel), nullptr);
+  if (!s) s = allow_shared(reinterpret_cast<const void*>(bisect_kernel), nullptr);
+  if (!s) s = allow_shared(reinterpret_cast<const void*>(k2), nullptr);
+  if (s) return s;
+  const size_t smem = sizeof(double) * team_doubles(A.nu);
+  k1<<<(unsigned)((A.n_cols + C1 - 1) / C1), 32, smem * C1, st>>>(A);
+  if (A.n_cols <= kFewColumns)
+    bisect_kernel<<<(unsigned)(A.n_cols * ((A.nu + 31) / 32)), 32, sizeof(double) * 2 * A.nu, st>>>(A);
+  else
+    ql_kernel<<<(unsigned)((A.n_cols + 31) / 32), 32, sizeof(double) * 2 * A.nu * 32, st>>>(A);
+  k2<<<(unsigned)((A.n_cols + C2 - 1) / C2), 32, smem * C2, st>>>(A);
+  count_launches(3);
+  MKA_CUDA_TRY(cudaGetLastError());
+  return MKA_OK;
+}
+
+}  // namespace
 
 mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
                           double* w, double* cv, int64_t col0, cudaStream_t st) {

@@ -95,3 +95,23 @@ def test_subspaces_of_several_sizes(lib):
                 a = b
     finally:
         mka.mka_system_destroy(s)
+
+
+@pytest.mark.parametrize("p,q", [(8, 7), (10, 10)])
+def test_degenerate_levels(lib, p, q):
+    """A perfect crystal: the three p columns of an atom have the same levels, and a column's own come close together.
+    Few columns (bisection) against the same in a selection above 2,048 (QL)."""
+    mka = lib
+    pos, box = lattice_positions("diamond", 3.567, 5, 0.0, 0.0, 1)
+    s = mka.mka_build_system(pos, box, SK_CARBON_LIKE, "fp64", cluster_radius=5.0)
+    try:
+        few = levels(mka, s, np.array([7], dtype=np.int64), p, q)
+        many = levels(mka, s, np.arange(600, dtype=np.int64), p, q)
+        np.testing.assert_array_equal(many["nu_eff"][28:32], few["nu_eff"])
+        np.testing.assert_allclose(many["eps"][28:32], few["eps"], rtol=0, atol=TOL)
+        for c in range(4):      # weights of levels closer than the tolerance may mix: compare their running sums
+            a, b = np.cumsum(many["w"][28 + c]), np.cumsum(few["w"][c])
+            apart = np.append(np.diff(few["eps"][c]) > 1e-6, True)
+            np.testing.assert_allclose(a[apart], b[apart], rtol=0, atol=TOL)
+    finally:
+        mka.mka_system_destroy(s)
