@@ -84,9 +84,10 @@ __device__ __forceinline__ double mi_comp(double pb, double pa, double L, double
 
 // One warp per atom; per warp kFeatGather (distance, id) candidate slots in shared memory.
 __global__ void __launch_bounds__(256) features_kernel(FeatArgs A) {
-  __shared__ double rk[8][kFeatGather];
+  __shared__ unsigned long long rk[8][kFeatGather];   // bits of the distance
   __shared__ int idk[8][kFeatGather];
   __shared__ int cnt[8];
+  __shared__ int near[8][kNeigh];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t warp = (int64_t)blockIdx.x * 8 + wid, nw = (int64_t)gridDim.x * 8;
   for (int64_t t = warp; t < A.n_sel; t += nw) {
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(256) features_kernel(FeatArgs A) {
         if (r2 <= A.r_gather2) {
           const int s = atomicAdd(&cnt[wid], 1);
           if (s < kFeatGather) {
-            rk[wid][s] = __dsqrt_rn(r2);
+            rk[wid][s] = (unsigned long long)__double_as_longlong(__dsqrt_rn(r2));
             idk[wid][s] = b;
           }
         }
@@ -128,47 +129,38 @@ __global__ void __launch_bounds__(256) features_kernel(FeatArgs A) {
     }
     __syncwarp();
     const int n = min(cnt[wid], kFeatGather);
+    // the 32 nearest by (distance, id): a candidate's place is the number of candidates before it, counted on the bits
+    // of the distances, whose order as integers is their own (none is negative). Repeated minima took 32 rounds of FP64
+    // compares and shuffles, 2.27 ms for 13,824 atoms.
+    if (lane < kNeigh) near[wid][lane] = -1;
+    __syncwarp();
+    for (int s0 = lane; s0 < n; s0 += 32) {
+      const unsigned long long r = rk[wid][s0];
+      const int id = idk[wid][s0];
+      int before = 0;
+      for (int s = 0; s < n; ++s) {
+        const unsigned long long rs = rk[wid][s];
+        before += rs < r || (rs == r && idk[wid][s] < id);
+      }
+      if (before < kNeigh) near[wid][before] = s0;
+    }
+    __syncwarp();
     float geo[4] = {0, 0, 0, 0};   // lane k < 32 keeps neighbour k's (d, l, m, n)
     int my_id = -1;
-    // the 32 nearest by repeated warp minima of (distance, id)
-    for (int k = 0; k < kNeigh; ++k) {
-      double best = INFINITY;
-      int bid = 0x7fffffff, bi = -1;
-      for (int s = lane; s < n; s += 32) {
-        const double r = rk[wid][s];
-        const int id = idk[wid][s];
-        if (r < best || (r == best && id < bid)) {
-          best = r;
-          bid = id;
-          bi = s;
-        }
+    const int bi = near[wid][lane];
+    if (bi >= 0) {
+      const int bid = idk[wid][bi];
+      const double best = __longlong_as_double((long long)rk[wid][bi]);
+      my_id = bid;
+      if (best <= 3.0) {
+        const double dx = mi_comp(A.pos[3 * bid], px, A.box[0], A.inv_box[0]);
+        const double dy = mi_comp(A.pos[3 * bid + 1], py, A.box[1], A.inv_box[1]);
+        const double dz = mi_comp(A.pos[3 * bid + 2], pz, A.box[2], A.inv_box[2]);
+        geo[0] = (float)best;
+        geo[1] = (float)__ddiv_rn(dx, best);
+        geo[2] = (float)__ddiv_rn(dy, best);
+        geo[3] = (float)__ddiv_rn(dz, best);
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oid = __shfl_xor_sync(0xffffffffu, bid, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob < best || (ob == best && oid < bid)) {
-          best = ob;
-          bid = oid;
-          bi = oi;
-        }
-      }
-      if (bi < 0) break;
-      if (lane == k) {
-        my_id = bid;
-        if (best <= 3.0) {
-          const double dx = mi_comp(A.pos[3 * bid], px, A.box[0], A.inv_box[0]);
-          const double dy = mi_comp(A.pos[3 * bid + 1], py, A.box[1], A.inv_box[1]);
-          const double dz = mi_comp(A.pos[3 * bid + 2], pz, A.box[2], A.inv_box[2]);
-          geo[0] = (float)best;
-          geo[1] = (float)__ddiv_rn(dx, best);
-          geo[2] = (float)__ddiv_rn(dy, best);
-          geo[3] = (float)__ddiv_rn(dz, best);
-        }
-      }
-      __syncwarp();
-      if (lane == 0) rk[wid][bi] = INFINITY;
-      __syncwarp();
     }
     for (int o = 0; o < 4; ++o) {
       float* row = A.X + (4 * t + o) * (int64_t)kIn;
