@@ -1180,7 +1180,7 @@ mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_para
   int32_t* patch = nullptr;
   const int64_t rows_max = 4 * std::min(res->n_sel, chunk);
   if (prm->use_warm_start) {
-    MKA_CUDA_TRY(cudaMallocAsync(&wbuf, sizeof(float) * (rows_max * (132 + 68) + mlp_work_floats(rows_max)), st));
+    MKA_CUDA_TRY(cudaMallocAsync(&wbuf, sizeof(float) * rows_max * (132 + 68), st));
     MKA_CUDA_TRY(cudaMallocAsync(&patch, sizeof(int32_t) * 17 * std::min(res->n_sel, chunk), st));
   }
   for (int64_t off = 0; off < res->n_sel && !s; off += chunk) {
@@ -1190,9 +1190,8 @@ mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_para
       const int64_t rows = 4 * cnt;
       float* X = wbuf;
       float* Y = X + rows * 132;
-      float* W = Y + rows * 68;
       s = features_enqueue(sys, res->d_sel + off, cnt, X, patch, st);
-      if (!s) s = mlp_forward_enqueue(sys->warm, X, rows, W, W + rows * 128, W + 2 * rows * 128, W + 3 * rows * 128, Y, st);
+      if (!s) s = mlp_forward_enqueue(sys->warm, X, rows, Y, st);
       if (s) break;
       a.x0 = Y;
       a.patch = patch;

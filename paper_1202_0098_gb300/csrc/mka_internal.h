@@ -172,9 +172,7 @@ mka_status reduced_launch(double* red, int64_t n_cols, int nu, int32_t* status, 
 // Learned warm start (mlp.cu).
 mka_status features_enqueue(const mka_system* sys, const int64_t* d_sel, int64_t n, float* X, int32_t* patch,
                             cudaStream_t st);
-mka_status mlp_forward_enqueue(const mka_mlp* net, const float* X, int64_t B, float* Z1, float* H1, float* Z2,
-                               float* H2, float* Y, cudaStream_t st);
-int64_t mlp_work_floats(int64_t B);   // floats of forward/backward work buffers for B rows
+mka_status mlp_forward_enqueue(const mka_mlp* net, const float* X, int64_t B, float* Y, cudaStream_t st);
 
 // What the per-atom kernels are configured for.
 struct AtomsShape {

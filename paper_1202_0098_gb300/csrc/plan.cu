@@ -143,7 +143,7 @@ mka_status plan_alloc(mka_plan* P) {
   MKA_CUDA_TRY(cudaEventCreate(&P->k2));
   if (P->prm.use_warm_start) {
     MKA_CUDA_TRY(cudaMalloc(&r->d_fallback, sizeof(int32_t) * 4 * A));
-    MKA_CUDA_TRY(cudaMalloc(&P->warm, sizeof(float) * (4 * A * (132 + 68) + mlp_work_floats(4 * A))));
+    MKA_CUDA_TRY(cudaMalloc(&P->warm, sizeof(float) * 4 * A * (132 + 68)));
     MKA_CUDA_TRY(cudaMalloc(&P->patch, sizeof(int32_t) * 17 * A));
   }
   return MKA_OK;
@@ -175,9 +175,8 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
     const int64_t rows = 4 * n;
     float* X = P->warm;
     float* Y = X + 4 * P->max_atoms * 132;
-    float* W = Y + 4 * P->max_atoms * 68;
     mka_status sw = features_enqueue(P->sys, r->d_sel, n, X, P->patch, st);
-    if (!sw) sw = mlp_forward_enqueue(P->sys->warm, X, rows, W, W + rows * 128, W + 2 * rows * 128, W + 3 * rows * 128, Y, st);
+    if (!sw) sw = mlp_forward_enqueue(P->sys->warm, X, rows, Y, st);
     if (sw) return sw;
     a.x0 = Y;
     a.patch = P->patch;
