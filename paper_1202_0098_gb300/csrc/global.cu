@@ -18,9 +18,7 @@
 #include <algorithm>
 #include <cmath>
 
-#include "kept.cuh"
 #include "mka_internal.h"
-#include "widen.cuh"
 #include "mu_root.cuh"
 
 namespace mka {
@@ -169,19 +167,32 @@ __global__ void mu_init_kernel(RootState* S, unsigned* ticket, double target, do
 
 __global__ void mu_finish_kernel(const RootState* S, double* mu_out) { *mu_out = 0.5 * (S->lo + S->hi); }
 
+// Column c of atom t: g = C diag(x) V_j for per-level weights x (ascending order of eps), from the
+// kept C and V_j (lane-interleaved by column); thread per (c, n), g into shared memory [4][nu].
+__device__ void column_weights(const double* cv, int64_t t, int nu, const double* x, double* g) {
+  for (int i = threadIdx.x; i < 4 * nu; i += blockDim.x) {
+    const int c = i / nu, n = i % nu;
+    const int64_t col = 4 * t + c;
+    const double* b = cv + (size_t)(col >> 5) * kept_block_doubles(nu) * 32 + (col & 31);
+    double s = 0.0;
+    for (int a = 0; a < nu; ++a) s += b[(size_t)(n * nu + a) * 32] * x[c * nu + a] * b[(size_t)(nu * nu + a) * 32];
+    g[i] = s;
+  }
+  __syncthreads();
+}
+
 // rho / E: one CTA per selected atom, thread per (block k, c, r) of its row:
 // rho_ij = sum_alpha f_alpha V_i alpha V_j alpha = U_i . g_j with g_j = C diag(f) V_j.
 // Output layout: the batch's (blocks at blk_off[t], E of atom t at e_partial[t]) when out_base < 0;
 // otherwise the system's pattern order from block out_base on (blocks at row_ptr[atom] - out_base,
 // E at e_partial[atom - e_base]).
-__global__ void __launch_bounds__(128) density_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
+__global__ void density_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
                                const int64_t* sel, const int32_t* row_ptr, const void* valH, int storage,
                                int nu, double mu_host, const double* mu_dev, double kT, double* rho,
                                double* e_partial, int64_t out_base = -1, int64_t e_base = 0) {
   __shared__ double red[kRedThreads / 32];
-  extern __shared__ __align__(16) double sm[];     // g, f: 4 nu each
-  double *g = sm, *f = sm + 4 * nu;
-  const bool pair = rows_paired(vp, nu);
+  __shared__ double f[4 * MKA_MAX_NU];
+  __shared__ double g[4 * MKA_MAX_NU];
   const double mu = mu_dev ? *mu_dev : mu_host;
   const int64_t t = blockIdx.x;
   const int64_t atom = sel[t];
@@ -193,13 +204,13 @@ __global__ void __launch_bounds__(128) density_kernel(const double* vp, const do
     f[i] = fermi(eps[(4 * t + c) * nu + i % nu], mu, kT);
   }
   __syncthreads();
-  column_weights<1>(cv, t, nu, f, g);
+  column_weights(cv, t, nu, f, g);
   double e = 0.0;
   for (int i = threadIdx.x; i < nrow * 16; i += blockDim.x) {
     const int k = i >> 4, c = (i >> 2) & 3, r = i & 3;
     const double* u = vp + ((b0 + k) * 16 + c * 4 + r) * (int64_t)nu;
-    double s;
-    row_products<1>(u, g + c * nu, 0, nu, pair, &s);
+    double s = 0.0;
+    for (int n = 0; n < nu; ++n) s += u[n] * g[c * nu + n];
     if (rho) rho[(ob + k) * 16 + c * 4 + r] = s;
     const int64_t gk = (int64_t)row_ptr[atom] + k;
     double h;
@@ -213,11 +224,9 @@ __global__ void __launch_bounds__(128) density_kernel(const double* vp, const do
 }
 
 // G_ij(z) = sum_alpha V_i alpha V_j alpha / (z - eps_alpha) = U_i . (C diag(1 / (z - eps)) V_j).
-__global__ void __launch_bounds__(128) greens_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
+__global__ void greens_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
                               const int64_t* sel, const int32_t* row_ptr, int nu, double zr, double zi, double* g) {
-  extern __shared__ __align__(16) double sm[];     // g, x: real and imaginary parts, 4 nu each
-  double *gv = sm, *xr = sm + 8 * nu, *xi = xr + 4 * nu;
-  const bool pair = rows_paired(vp, nu);
+  __shared__ double xr[4 * MKA_MAX_NU], xi[4 * MKA_MAX_NU], gr[4 * MKA_MAX_NU], gi[4 * MKA_MAX_NU];
   const int64_t t = blockIdx.x;
   const int64_t atom = sel[t];
   const int nrow = row_ptr[atom + 1] - row_ptr[atom];
@@ -230,14 +239,18 @@ __global__ void __launch_bounds__(128) greens_kernel(const double* vp, const dou
     xi[i] = -zi / den;
   }
   __syncthreads();
-  column_weights<2>(cv, t, nu, xr, gv);
+  column_weights(cv, t, nu, xr, gr);
+  column_weights(cv, t, nu, xi, gi);
   for (int i = threadIdx.x; i < nrow * 16; i += blockDim.x) {
     const int k = i >> 4, c = (i >> 2) & 3, r = i & 3;
     const double* u = vp + ((b0 + k) * 16 + c * 4 + r) * (int64_t)nu;
-    double s[2];
-    row_products<2>(u, gv + c * nu, 4 * nu, nu, pair, s);
-    g[2 * ((b0 + k) * 16 + c * 4 + r)] = s[0];
-    g[2 * ((b0 + k) * 16 + c * 4 + r) + 1] = s[1];
+    double sr = 0.0, si = 0.0;
+    for (int n = 0; n < nu; ++n) {
+      sr += u[n] * gr[c * nu + n];
+      si += u[n] * gi[c * nu + n];
+    }
+    g[2 * ((b0 + k) * 16 + c * 4 + r)] = sr;
+    g[2 * ((b0 + k) * 16 + c * 4 + r) + 1] = si;
   }
 }
 
@@ -321,136 +334,51 @@ __device__ __forceinline__ void load_x(const TX* __restrict__ x, int64_t cb, TX 
   }
 }
 
-constexpr int kSpmvThreads = 128;
-// CTAs on an SM, which sets the registers: four atoms' values and x rows in flight at K = 1, more warps with two or one
-// (FP32 values and x, 262,144 atoms: K = 1 at 5 / 8 CTAs 50 / 68 us, K = 4 79 / 70).
-template <typename TX, int K>
-constexpr int kSpmvBlocks = sizeof(TX) == 8 ? (K == 1 ? 4 : 5) : (K == 1 ? 5 : 8);
-
-// A warp takes PER neighbouring atoms at a time: lane = (place, slot, row i), 8 / SLOTS places of 4 / K atoms each; the
-// lane has row i of the blocks slot, slot + SLOTS, ... of its place's atoms, so that a load takes whole blocks that lie
-// next to each other, and 4 / K atoms of K vectors are four sums a lane, which the slots halve among themselves. Warps
-// walk over the system with the next atoms' columns and row pointers loaded ahead, so that only one latency is left
-// between values and products.
-// Memory bounds FP32 and BF16 values, the FP64 pipe bounds FP64 vectors (stored FP32 values are widened by integer
-// operations: 275 -> 136 us at K = 1). A thread per row with its 13 blocks one after another: FP32, K = 1, 262,144 atoms
-// 57 us against 45 here (36 is the floor); 512 atoms, FP64, K = 4, on 8 SMs, 22.5 against 6.1.
-template <typename TV, typename TX, int K, int SLOTS>
-__global__ void __launch_bounds__(kSpmvThreads, (kSpmvBlocks<TX, K>))
-    spmv_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, const TV* __restrict__ val,
-                const TX* __restrict__ x, TX* __restrict__ y, int64_t n_rows) {
+template <typename TV, typename TX, int K>
+__global__ void __launch_bounds__(256) spmv_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+                                                   const TV* __restrict__ val, const TX* __restrict__ x,
+                                                   TX* __restrict__ y, int64_t n_rows) {
   using TL = typename std::conditional<std::is_same<TV, double>::value, double, float>::type;
-  constexpr int A = 4 / K, PER = A * (8 / SLOTS), R = 2;
-  constexpr bool kAhead = sizeof(TX) == 4;
-  const int lane = threadIdx.x & 31, i = lane & 3, slot = (lane >> 2) % SLOTS, place = lane / (4 * SLOTS);
-  const int64_t nw = (int64_t)gridDim.x * (kSpmvThreads / 32);
-  const int64_t groups = (n_rows + PER - 1) / PER;
-  int64_t g = ((int64_t)blockIdx.x * kSpmvThreads + threadIdx.x) >> 5;
-  if (g >= groups) return;
-  auto pointer = [&](int64_t gg) {      // lane l: row pointer of the group's atom l (the end beyond the last)
-    const int64_t a = gg * PER + (lane < PER ? lane : PER);
-    return gg < groups ? __ldg(row_ptr + (a < n_rows ? a : n_rows)) : 0;
-  };
-  int k0[A], k1[A], cb[A][R];
-  auto take = [&](int rp) {             // the lane's atoms of a group: bounds and first columns
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < 4 * n_rows; g += stride) {
+    const int64_t a = g >> 2;
+    const int i = (int)(g & 3);
+    const int k0 = __ldg(row_ptr + a), k1 = __ldg(row_ptr + a + 1);
+    TX acc[K];
 #pragma unroll
-    for (int u = 0; u < A; ++u) {
-      k0[u] = __shfl_sync(0xffffffffu, rp, place * A + u) + slot;
-      k1[u] = __shfl_sync(0xffffffffu, rp, place * A + u + 1);
+    for (int c = 0; c < K; ++c) acc[c] = 0;
+    int k = k0;
+    for (; k + 4 <= k1; k += 4) {
+      int cb[4];
+      TL v[4][4];
 #pragma unroll
-      for (int h = 0; h < R; ++h) cb[u][h] = k0[u] + SLOTS * h < k1[u] ? __ldg(col + k0[u] + SLOTS * h) : -1;
-    }
-  };
-  int rp = pointer(g), next = pointer(g + nw);
-  take(rp);
-  for (; g < groups; g += nw) {
-    TX s[4] = {0, 0, 0, 0};
-    for (bool first = true;; first = false) {
-      TL v[A][R][4];
-      int c[A][R];
-      bool more = false;
+      for (int u = 0; u < 4; ++u) cb[u] = __ldg(col + k + u);
 #pragma unroll
-      for (int u = 0; u < A; ++u) {
+      for (int u = 0; u < 4; ++u) RowVals<TV>::load(val, k + u, i, v[u]);
 #pragma unroll
-        for (int h = 0; h < R; ++h) {
-          c[u][h] = cb[u][h];
+      for (int u = 0; u < 4; ++u) {
+        TX xv[4][K];
+        load_x<TX, K>(x, cb[u], xv);
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) v[u][h][jj] = 0;
-          if (c[u][h] >= 0) RowVals<TV>::load(val, k0[u] + SLOTS * h, i, v[u][h]);
-        }
-        more = more || k0[u] + SLOTS * R < k1[u];
+        for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+          for (int c = 0; c < K; ++c) acc[c] = fma((TX)v[u][jj], xv[jj][c], acc[c]);
       }
-      const bool again = __any_sync(0xffffffffu, more);
-      if (again) {
-#pragma unroll
-        for (int u = 0; u < A; ++u) {
-          k0[u] = min(k0[u] + SLOTS * R, k1[u]);
-#pragma unroll
-          for (int h = 0; h < R; ++h) cb[u][h] = k0[u] + SLOTS * h < k1[u] ? __ldg(col + k0[u] + SLOTS * h) : -1;
-        }
-      } else {
-        take(next);
-        next = pointer(g + 2 * nw);
-      }
-      TX xs[A][R][4][K];                // FP32: all x rows in flight too; FP64 has not the registers, nor the need
-      if constexpr (kAhead) {
-#pragma unroll
-        for (int u = 0; u < A; ++u)
-#pragma unroll
-          for (int h = 0; h < R; ++h) {
-#pragma unroll
-            for (int e = 0; e < 4 * K; ++e) xs[u][h][e / K][e % K] = 0;
-            if (c[u][h] >= 0) load_x<TX, K>(x, c[u][h], xs[u][h]);
-          }
-      }
-#pragma unroll
-      for (int u = 0; u < A; ++u)
-#pragma unroll
-        for (int h = 0; h < R; ++h) {
-          TX (&xv)[4][K] = xs[u][h];
-          if constexpr (!kAhead) {
-            if (c[u][h] < 0) continue;
-            load_x<TX, K>(x, c[u][h], xv);
-          }
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            TX w;
-            if constexpr (sizeof(TX) > sizeof(TL)) w = widen(v[u][h][jj]);
-            else w = (TX)v[u][h][jj];
-#pragma unroll
-            for (int q = 0; q < K; ++q) s[u * K + q] = fma(w, xv[jj][q], s[u * K + q]);
-          }
-        }
-      if (!again) break;
     }
-    TX t[2];
-    if constexpr (SLOTS == 8) {
-      const int hi = lane >> 4 & 1, lo = lane >> 3 & 1;
+    for (; k < k1; ++k) {
+      TL v[4];
+      RowVals<TV>::load(val, k, i, v);
+      TX xv[4][K];
+      load_x<TX, K>(x, __ldg(col + k), xv);
 #pragma unroll
-      for (int q = 0; q < 2; ++q) t[q] = (hi ? s[2 + q] : s[q]) + __shfl_xor_sync(0xffffffffu, hi ? s[q] : s[2 + q], 16);
-      TX r = (lo ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, lo ? t[0] : t[1], 8);
-      r += __shfl_xor_sync(0xffffffffu, r, 4);
-      const int e = 2 * hi + lo;                  // atom e / K of the group, vector e % K
-      const int64_t a = g * PER + e / K;
-      if ((slot & 1) == 0 && a < n_rows) y[(4 * a + i) * K + e % K] = r;
-    } else {
-      const int hi = lane >> 3 & 1, lo = lane >> 2 & 1;
+      for (int jj = 0; jj < 4; ++jj)
 #pragma unroll
-      for (int q = 0; q < 2; ++q) t[q] = (hi ? s[2 + q] : s[q]) + __shfl_xor_sync(0xffffffffu, hi ? s[q] : s[2 + q], 8);
-      const TX r = (lo ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, lo ? t[0] : t[1], 4);
-      const int e = 2 * hi + lo;
-      const int64_t a = g * PER + place * A + e / K;
-      if (a < n_rows) y[(4 * a + i) * K + e % K] = r;
+        for (int c = 0; c < K; ++c) acc[c] = fma((TX)v[jj], xv[jj][c], acc[c]);
     }
+    TX* yo = y + (4 * a + i) * K;
+#pragma unroll
+    for (int c = 0; c < K; ++c) yo[c] = acc[c];
   }
-}
-
-template <typename TV, typename TX, int K, int SLOTS>
-void spmv_launch(const mka_system* s, const TV* val, const TX* x, TX* y, int sms, cudaStream_t st) {
-  const int64_t per = (int64_t)(4 / K) * (8 / SLOTS) * (kSpmvThreads / 32);
-  const int64_t blocks = std::min<int64_t>((s->n_atoms + per - 1) / per, (int64_t)sms * kSpmvBlocks<TX, K>);
-  spmv_kernel<TV, TX, K, SLOTS><<<(unsigned)std::max<int64_t>(1, blocks), kSpmvThreads, 0, st>>>(
-      s->d_row_ptr, s->d_col, val, x, y, s->n_atoms);
 }
 
 template <typename TV, typename TX>
@@ -458,15 +386,12 @@ mka_status spmv_dispatch_k(const mka_system* s, const TV* val, const void* x, vo
   int dev = 0, sms = 0;
   MKA_CUDA_TRY(cudaGetDevice(&dev));
   MKA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((4 * s->n_atoms + 255) / 256, (int64_t)sms * 8));
   const TX* xx = reinterpret_cast<const TX*>(x);
   TX* yy = reinterpret_cast<TX*>(y);
-  // Four slots waste less on rows of 13 blocks and add less (FP64, K = 4, 262,144 atoms: 492 against 539 us); eight spread
-  // a small system over more warps (512 atoms, K = 4: 8.8 against 10.9 us; 4,096 atoms, K = 1: 12.9 against 15). They meet at
-  // about eight warps an SM.
-  const bool wide = s->n_atoms * k < (int64_t)sms * 64;
-  if (k == 1) wide ? spmv_launch<TV, TX, 1, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 1, 4>(s, val, xx, yy, sms, st);
-  else if (k == 2) wide ? spmv_launch<TV, TX, 2, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 2, 4>(s, val, xx, yy, sms, st);
-  else wide ? spmv_launch<TV, TX, 4, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 4, 4>(s, val, xx, yy, sms, st);
+  if (k == 1) spmv_kernel<TV, TX, 1><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
+  else if (k == 2) spmv_kernel<TV, TX, 2><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
+  else spmv_kernel<TV, TX, 4><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
@@ -484,7 +409,7 @@ mka_status spmv_dispatch(const mka_system* s, const void* val, int x_dtype, cons
 // a time; its 8 warps take 8 groups of 32 energies, or, with fewer groups than warps, share a group's levels among
 // them (interleaved, added in warp order), so that 41 energies do not leave 7 of 8 lanes idle. A second kernel
 // adds the chunk sums in a fixed order, a warp per energy. FP64 throughout; the divisions bound it. The chunk grows with
-// the levels: 32,768 levels a chunk left 14,800 levels to one CTA (12.1 ms for 201 energies, now under 0.3 ms).
+// the levels: 32,768 levels a chunk left 14,800 levels to one CTA (12.1 ms for 201 energies).
 constexpr int kDosThreads = 256, kDosWarps = kDosThreads / 32;
 
 __global__ void __launch_bounds__(kDosThreads) dos_partial_kernel(const double* eps, const double* w, int64_t n,
@@ -623,7 +548,7 @@ mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n_cols, i
 mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int64_t* blk_off, const double* vp,
                            const double* cv, const double* eps, const double* w, int64_t n_sel, int nu,
                            const double* mu_dev, double kT, double* rho_out, double* tmp, cudaStream_t st) {
-  density_kernel<<<(unsigned)n_sel, 128, sizeof(double) * 8 * nu, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH,
+  density_kernel<<<(unsigned)n_sel, 128, 0, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH,
                                                   sys->storage, nu, 0.0, mu_dev, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, n_sel, tmp + n_sel);
   const int rb = red_blocks();
@@ -637,7 +562,7 @@ mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int6
 mka_status density_global_enqueue(const mka_system* sys, const int64_t* sel, const int64_t* blk_off, const double* vp,
                                   const double* cv, const double* eps, int64_t n_sel, int nu, double mu, double kT,
                                   double* rho, int64_t out_base, double* e_atom, int64_t e_base, cudaStream_t st) {
-  density_kernel<<<(unsigned)n_sel, 128, sizeof(double) * 8 * nu, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH, sys->storage,
+  density_kernel<<<(unsigned)n_sel, 128, 0, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH, sys->storage,
                                                   nu, mu, nullptr, kT, rho, e_atom, out_base, e_base);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
@@ -682,7 +607,7 @@ mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT
   double* tmp = nullptr;
   const int rb = red_blocks();
   MKA_CUDA_TRY(cudaMallocAsync(&tmp, sizeof(double) * (res->n_sel + 2 + rb), st));
-  density_kernel<<<(unsigned)res->n_sel, 128, sizeof(double) * 8 * res->nu, st>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
+  density_kernel<<<(unsigned)res->n_sel, 128, 0, st>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
                                                        res->d_sel, sys->d_row_ptr, sys->d_valH, sys->storage,
                                                        res->nu, mu, nullptr, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, res->n_sel, tmp + res->n_sel);
@@ -706,7 +631,7 @@ mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT
 }
 
 mka_status launch_greens(mka_system* sys, mka_result* res, double z_re, double z_im, double* g_out) {
-  greens_kernel<<<(unsigned)res->n_sel, 128, sizeof(double) * 16 * res->nu, res->stream>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
+  greens_kernel<<<(unsigned)res->n_sel, 128, 0, res->stream>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
                                                                res->d_sel, sys->d_row_ptr, res->nu, z_re, z_im, g_out);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
