@@ -11,8 +11,10 @@
 // derivative of the exact model; values may be stored rounded).
 //
 // force_blocks_kernel: one CTA per selected atom b, thread per pattern entry (k, c, r):
-//   rho = U_i . (C diag(f) V_j), pi = U_i . (C diag(f eps) V_j) from the kept data, then the entry's
-//   three contributions, summed over the block's 16 entries by a fixed xor tree, one 3-vector per block.
+//   rho = U_i . (C diag(f) V_j), pi = U_i . (C diag(f eps) V_j) from the kept data; then a thread per pattern
+//   block contracts its 16 entries of each with the block's derivative, one 3-vector per block. The FP64 pipe bounds it:
+//   2 nu FMAs an entry and 2 nu an element row of C (2,048 atoms, nu = 30, 28,700 blocks: 348 -> 145 us with the derivatives
+//   contracted by block and C read in whole sectors; 74 us of it are those FMAs).
 // force_gather_kernel: F_K = sum over K's row blocks k' (neighbour a') of g[block of a' pointing to K]
 //   - g[k'], each looked up in a fixed order, so the forces do not depend on timing.
 #include <cuda_bf16.h>
@@ -22,6 +24,7 @@
 
 #include <algorithm>
 
+#include "kept.cuh"
 #include "mka_internal.h"
 #include "sk_grad.cuh"
 
@@ -57,66 +60,51 @@ struct ForceBlockArgs {
   double* g;                 // [blocks][3]
 };
 
-__global__ void __launch_bounds__(128) force_blocks_kernel(const ForceBlockArgs A) {
-  __shared__ double f[4 * MKA_MAX_NU], fe[4 * MKA_MAX_NU];
-  __shared__ double gr[4 * MKA_MAX_NU], gp[4 * MKA_MAX_NU];
+constexpr int kForceThreads = 128, kForceBlocks = 32;   // threads of a CTA; pattern blocks it takes at a time
+
+__global__ void __launch_bounds__(kForceThreads) force_blocks_kernel(const ForceBlockArgs A) {
+  extern __shared__ __align__(16) double sm[];    // g = C diag(x) V_j and x for x = f, f eps: 8 nu each; rho, pi
   const int nu = A.nu;
+  double *gv = sm, *f = sm + 8 * nu, *fe = f + 4 * nu;
+  double *s_rho = sm + 16 * nu, *s_pi = s_rho + 17 * kForceBlocks;
   const int64_t t = blockIdx.x;
   const int64_t atom = A.sel[t];
   const int64_t k0 = A.row_ptr[atom];
   const int nrow = A.row_ptr[atom + 1] - (int)k0;
   const int64_t b0 = A.blk_off[t];
   const int64_t ob = A.out_base < 0 ? b0 : k0 - A.out_base;
-  for (int i = threadIdx.x; i < 4 * nu; i += blockDim.x) {
-    const double e = A.eps[(4 * t + i / nu) * nu + i % nu];
+  for (int i = threadIdx.x; i < 4 * nu; i += kForceThreads) {
+    const double e = A.eps[4 * t * nu + i];
     f[i] = fermi_d(e, A.mu, A.kT);
     fe[i] = f[i] * e;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 4 * nu; i += blockDim.x) {   // g = C diag(x) V_j for x = f and f eps
-    const int c = i / nu, n = i % nu;
-    const int64_t colj = 4 * t + c;
-    const double* bk = A.cv + (size_t)(colj >> 5) * kept_block_doubles(nu) * 32 + (colj & 31);
-    double s1 = 0.0, s2 = 0.0;
-    for (int a = 0; a < nu; ++a) {
-      const double cv = bk[(size_t)(n * nu + a) * 32] * bk[(size_t)(nu * nu + a) * 32];
-      s1 += cv * f[c * nu + a];
-      s2 += cv * fe[c * nu + a];
-    }
-    gr[i] = s1;
-    gp[i] = s2;
-  }
-  __syncthreads();
+  column_weights<2>(A.cv, t, nu, f, gv);
   const double ax = A.pos[3 * atom], ay = A.pos[3 * atom + 1], az = A.pos[3 * atom + 2];
-  for (int base = 0; base < nrow * 16; base += blockDim.x) {   // whole warps iterate together (shuffles below)
-    const int i = base + threadIdx.x;
-    const bool on = i < nrow * 16;
-    const int k = i >> 4, c = (i >> 2) & 3, r = i & 3;
-    double e[3] = {0.0, 0.0, 0.0};
-    if (on) {
-      const double* u = A.vp + ((b0 + k) * 16 + c * 4 + r) * (int64_t)nu;
-      double rho = 0.0, pi = 0.0;
-      for (int n = 0; n < nu; ++n) {
-        rho += u[n] * gr[c * nu + n];
-        pi += u[n] * gp[c * nu + n];
-      }
-      if (A.pi) A.pi[(ob + k) * 16 + c * 4 + r] = pi;
-      const int64_t a = A.col[k0 + k];
+  const bool pair = rows_paired(A.vp, nu);
+  for (int kb = 0; kb < nrow; kb += kForceBlocks) {
+    const int nk = min(kForceBlocks, nrow - kb);
+    for (int i = threadIdx.x; i < nk * 16; i += kForceThreads) {
+      const int k = i >> 4, c = (i >> 2) & 3;
+      double s[2];
+      row_products<2>(A.vp + ((b0 + kb) * 16 + i) * (int64_t)nu, gv + c * nu, 4 * nu, nu, pair, s);
+      s_rho[17 * k + (i & 15)] = s[0];
+      s_pi[17 * k + (i & 15)] = s[1];
+      if (A.pi) A.pi[(ob + kb) * 16 + i] = s[1];
+    }
+    __syncthreads();
+    if (threadIdx.x < nk) {
+      const int k = threadIdx.x;
+      const int64_t a = A.col[k0 + kb + k];
+      double e[3] = {0.0, 0.0, 0.0};
       if (a != atom) {
         double d[3] = {A.pos[3 * a] - ax, A.pos[3 * a + 1] - ay, A.pos[3 * a + 2] - az};
         for (int q = 0; q < 3; ++q) d[q] -= A.box[q] * rint(d[q] / A.box[q]);
-        double gh[3], gs[3];
-        sk_entry_grad(d, A.Vh, A.d0, c, r, gh);
-        sk_entry_grad(d, A.Vs, A.d0, c, r, gs);
-        for (int q = 0; q < 3; ++q) e[q] = -2.0 * (rho * gh[q] - pi * gs[q]);
+        sk_block_force(d, A.Vh, A.Vs, A.d0, s_rho + 17 * k, s_pi + 17 * k, e);
       }
+      for (int q = 0; q < 3; ++q) A.g[(ob + kb + k) * 3 + q] = e[q];
     }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) e[q] += __shfl_xor_sync(0xffffffffu, e[q], o);
-    if (on && (threadIdx.x & 15) == 0)
-      for (int q = 0; q < 3; ++q) A.g[(ob + k) * 3 + q] = e[q];
+    __syncthreads();
   }
 }
 
@@ -190,7 +178,7 @@ mka_status force_blocks_enqueue(const mka_system* sys, const int64_t* sel, const
   A.out_base = out_base;
   A.pi = pi;
   A.g = g;
-  force_blocks_kernel<<<(unsigned)n_sel, 128, 0, st>>>(A);
+  force_blocks_kernel<<<(unsigned)n_sel, kForceThreads, sizeof(double) * (16 * nu + 2 * 17 * kForceBlocks), st>>>(A);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;

@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "kept.cuh"
 #include "mka_internal.h"
 #include "mu_root.cuh"
 
@@ -167,32 +168,19 @@ __global__ void mu_init_kernel(RootState* S, unsigned* ticket, double target, do
 
 __global__ void mu_finish_kernel(const RootState* S, double* mu_out) { *mu_out = 0.5 * (S->lo + S->hi); }
 
-// Column c of atom t: g = C diag(x) V_j for per-level weights x (ascending order of eps), from the
-// kept C and V_j (lane-interleaved by column); thread per (c, n), g into shared memory [4][nu].
-__device__ void column_weights(const double* cv, int64_t t, int nu, const double* x, double* g) {
-  for (int i = threadIdx.x; i < 4 * nu; i += blockDim.x) {
-    const int c = i / nu, n = i % nu;
-    const int64_t col = 4 * t + c;
-    const double* b = cv + (size_t)(col >> 5) * kept_block_doubles(nu) * 32 + (col & 31);
-    double s = 0.0;
-    for (int a = 0; a < nu; ++a) s += b[(size_t)(n * nu + a) * 32] * x[c * nu + a] * b[(size_t)(nu * nu + a) * 32];
-    g[i] = s;
-  }
-  __syncthreads();
-}
-
 // rho / E: one CTA per selected atom, thread per (block k, c, r) of its row:
 // rho_ij = sum_alpha f_alpha V_i alpha V_j alpha = U_i . g_j with g_j = C diag(f) V_j.
 // Output layout: the batch's (blocks at blk_off[t], E of atom t at e_partial[t]) when out_base < 0;
 // otherwise the system's pattern order from block out_base on (blocks at row_ptr[atom] - out_base,
 // E at e_partial[atom - e_base]).
-__global__ void density_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
+__global__ void __launch_bounds__(128) density_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
                                const int64_t* sel, const int32_t* row_ptr, const void* valH, int storage,
                                int nu, double mu_host, const double* mu_dev, double kT, double* rho,
                                double* e_partial, int64_t out_base = -1, int64_t e_base = 0) {
   __shared__ double red[kRedThreads / 32];
-  __shared__ double f[4 * MKA_MAX_NU];
-  __shared__ double g[4 * MKA_MAX_NU];
+  extern __shared__ __align__(16) double sm[];     // g, f: 4 nu each
+  double *g = sm, *f = sm + 4 * nu;
+  const bool pair = rows_paired(vp, nu);
   const double mu = mu_dev ? *mu_dev : mu_host;
   const int64_t t = blockIdx.x;
   const int64_t atom = sel[t];
@@ -204,13 +192,13 @@ __global__ void density_kernel(const double* vp, const double* cv, const double*
     f[i] = fermi(eps[(4 * t + c) * nu + i % nu], mu, kT);
   }
   __syncthreads();
-  column_weights(cv, t, nu, f, g);
+  column_weights<1>(cv, t, nu, f, g);
   double e = 0.0;
   for (int i = threadIdx.x; i < nrow * 16; i += blockDim.x) {
     const int k = i >> 4, c = (i >> 2) & 3, r = i & 3;
     const double* u = vp + ((b0 + k) * 16 + c * 4 + r) * (int64_t)nu;
-    double s = 0.0;
-    for (int n = 0; n < nu; ++n) s += u[n] * g[c * nu + n];
+    double s;
+    row_products<1>(u, g + c * nu, 0, nu, pair, &s);
     if (rho) rho[(ob + k) * 16 + c * 4 + r] = s;
     const int64_t gk = (int64_t)row_ptr[atom] + k;
     double h;
@@ -224,9 +212,11 @@ __global__ void density_kernel(const double* vp, const double* cv, const double*
 }
 
 // G_ij(z) = sum_alpha V_i alpha V_j alpha / (z - eps_alpha) = U_i . (C diag(1 / (z - eps)) V_j).
-__global__ void greens_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
+__global__ void __launch_bounds__(128) greens_kernel(const double* vp, const double* cv, const double* eps, const int64_t* blk_off,
                               const int64_t* sel, const int32_t* row_ptr, int nu, double zr, double zi, double* g) {
-  __shared__ double xr[4 * MKA_MAX_NU], xi[4 * MKA_MAX_NU], gr[4 * MKA_MAX_NU], gi[4 * MKA_MAX_NU];
+  extern __shared__ __align__(16) double sm[];     // g, x: real and imaginary parts, 4 nu each
+  double *gv = sm, *xr = sm + 8 * nu, *xi = xr + 4 * nu;
+  const bool pair = rows_paired(vp, nu);
   const int64_t t = blockIdx.x;
   const int64_t atom = sel[t];
   const int nrow = row_ptr[atom + 1] - row_ptr[atom];
@@ -239,18 +229,14 @@ __global__ void greens_kernel(const double* vp, const double* cv, const double* 
     xi[i] = -zi / den;
   }
   __syncthreads();
-  column_weights(cv, t, nu, xr, gr);
-  column_weights(cv, t, nu, xi, gi);
+  column_weights<2>(cv, t, nu, xr, gv);
   for (int i = threadIdx.x; i < nrow * 16; i += blockDim.x) {
     const int k = i >> 4, c = (i >> 2) & 3, r = i & 3;
     const double* u = vp + ((b0 + k) * 16 + c * 4 + r) * (int64_t)nu;
-    double sr = 0.0, si = 0.0;
-    for (int n = 0; n < nu; ++n) {
-      sr += u[n] * gr[c * nu + n];
-      si += u[n] * gi[c * nu + n];
-    }
-    g[2 * ((b0 + k) * 16 + c * 4 + r)] = sr;
-    g[2 * ((b0 + k) * 16 + c * 4 + r) + 1] = si;
+    double s[2];
+    row_products<2>(u, gv + c * nu, 4 * nu, nu, pair, s);
+    g[2 * ((b0 + k) * 16 + c * 4 + r)] = s[0];
+    g[2 * ((b0 + k) * 16 + c * 4 + r) + 1] = s[1];
   }
 }
 
@@ -409,7 +395,7 @@ mka_status spmv_dispatch(const mka_system* s, const void* val, int x_dtype, cons
 // a time; its 8 warps take 8 groups of 32 energies, or, with fewer groups than warps, share a group's levels among
 // them (interleaved, added in warp order), so that 41 energies do not leave 7 of 8 lanes idle. A second kernel
 // adds the chunk sums in a fixed order, a warp per energy. FP64 throughout; the divisions bound it. The chunk grows with
-// the levels: 32,768 levels a chunk left 14,800 levels to one CTA (12.1 ms for 201 energies).
+// the levels: 32,768 levels a chunk left 14,800 levels to one CTA (12.1 ms for 201 energies, 0.11 with the chip full).
 constexpr int kDosThreads = 256, kDosWarps = kDosThreads / 32;
 
 __global__ void __launch_bounds__(kDosThreads) dos_partial_kernel(const double* eps, const double* w, int64_t n,
@@ -548,7 +534,7 @@ mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n_cols, i
 mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int64_t* blk_off, const double* vp,
                            const double* cv, const double* eps, const double* w, int64_t n_sel, int nu,
                            const double* mu_dev, double kT, double* rho_out, double* tmp, cudaStream_t st) {
-  density_kernel<<<(unsigned)n_sel, 128, 0, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH,
+  density_kernel<<<(unsigned)n_sel, 128, sizeof(double) * 8 * nu, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH,
                                                   sys->storage, nu, 0.0, mu_dev, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, n_sel, tmp + n_sel);
   const int rb = red_blocks();
@@ -562,7 +548,7 @@ mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int6
 mka_status density_global_enqueue(const mka_system* sys, const int64_t* sel, const int64_t* blk_off, const double* vp,
                                   const double* cv, const double* eps, int64_t n_sel, int nu, double mu, double kT,
                                   double* rho, int64_t out_base, double* e_atom, int64_t e_base, cudaStream_t st) {
-  density_kernel<<<(unsigned)n_sel, 128, 0, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH, sys->storage,
+  density_kernel<<<(unsigned)n_sel, 128, sizeof(double) * 8 * nu, st>>>(vp, cv, eps, blk_off, sel, sys->d_row_ptr, sys->d_valH, sys->storage,
                                                   nu, mu, nullptr, kT, rho, e_atom, out_base, e_base);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
@@ -607,7 +593,7 @@ mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT
   double* tmp = nullptr;
   const int rb = red_blocks();
   MKA_CUDA_TRY(cudaMallocAsync(&tmp, sizeof(double) * (res->n_sel + 2 + rb), st));
-  density_kernel<<<(unsigned)res->n_sel, 128, 0, st>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
+  density_kernel<<<(unsigned)res->n_sel, 128, sizeof(double) * 8 * res->nu, st>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
                                                        res->d_sel, sys->d_row_ptr, sys->d_valH, sys->storage,
                                                        res->nu, mu, nullptr, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, res->n_sel, tmp + res->n_sel);
@@ -631,7 +617,7 @@ mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT
 }
 
 mka_status launch_greens(mka_system* sys, mka_result* res, double z_re, double z_im, double* g_out) {
-  greens_kernel<<<(unsigned)res->n_sel, 128, 0, res->stream>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
+  greens_kernel<<<(unsigned)res->n_sel, 128, sizeof(double) * 16 * res->nu, res->stream>>>(res->d_vp, res->d_cv, res->d_eps, res->d_blk_off,
                                                                res->d_sel, sys->d_row_ptr, res->nu, z_re, z_im, g_out);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
