@@ -20,6 +20,7 @@
 
 #include "kept.cuh"
 #include "mka_internal.h"
+#include "widen.cuh"
 #include "mu_root.cuh"
 
 namespace mka {
@@ -320,51 +321,136 @@ __device__ __forceinline__ void load_x(const TX* __restrict__ x, int64_t cb, TX 
   }
 }
 
-template <typename TV, typename TX, int K>
-__global__ void __launch_bounds__(256) spmv_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                                                   const TV* __restrict__ val, const TX* __restrict__ x,
-                                                   TX* __restrict__ y, int64_t n_rows) {
+constexpr int kSpmvThreads = 128;
+// CTAs on an SM, which sets the registers: four atoms' values and x rows in flight at K = 1, more warps with two or one
+// (FP32 values and x, 262,144 atoms: K = 1 at 5 / 8 CTAs 50 / 68 us, K = 4 79 / 70).
+template <typename TX, int K>
+constexpr int kSpmvBlocks = sizeof(TX) == 8 ? (K == 1 ? 4 : 5) : (K == 1 ? 5 : 8);
+
+// A warp takes PER neighbouring atoms at a time: lane = (place, slot, row i), 8 / SLOTS places of 4 / K atoms each; the
+// lane has row i of the blocks slot, slot + SLOTS, ... of its place's atoms, so that a load takes whole blocks that lie
+// next to each other, and 4 / K atoms of K vectors are four sums a lane, which the slots halve among themselves. Warps
+// walk over the system with the next atoms' columns and row pointers loaded ahead, so that only one latency is left
+// between values and products.
+// Memory bounds FP32 and BF16 values, the FP64 pipe bounds FP64 vectors (stored FP32 values are widened by integer
+// operations: 275 -> 136 us at K = 1). A thread per row with its 13 blocks one after another: FP32, K = 1, 262,144 atoms
+// 57 us against 45 here (36 is the floor); 512 atoms, FP64, K = 4, on 8 SMs, 22.5 against 6.1.
+template <typename TV, typename TX, int K, int SLOTS>
+__global__ void __launch_bounds__(kSpmvThreads, (kSpmvBlocks<TX, K>))
+    spmv_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, const TV* __restrict__ val,
+                const TX* __restrict__ x, TX* __restrict__ y, int64_t n_rows) {
   using TL = typename std::conditional<std::is_same<TV, double>::value, double, float>::type;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < 4 * n_rows; g += stride) {
-    const int64_t a = g >> 2;
-    const int i = (int)(g & 3);
-    const int k0 = __ldg(row_ptr + a), k1 = __ldg(row_ptr + a + 1);
-    TX acc[K];
+  constexpr int A = 4 / K, PER = A * (8 / SLOTS), R = 2;
+  constexpr bool kAhead = sizeof(TX) == 4;
+  const int lane = threadIdx.x & 31, i = lane & 3, slot = (lane >> 2) % SLOTS, place = lane / (4 * SLOTS);
+  const int64_t nw = (int64_t)gridDim.x * (kSpmvThreads / 32);
+  const int64_t groups = (n_rows + PER - 1) / PER;
+  int64_t g = ((int64_t)blockIdx.x * kSpmvThreads + threadIdx.x) >> 5;
+  if (g >= groups) return;
+  auto pointer = [&](int64_t gg) {      // lane l: row pointer of the group's atom l (the end beyond the last)
+    const int64_t a = gg * PER + (lane < PER ? lane : PER);
+    return gg < groups ? __ldg(row_ptr + (a < n_rows ? a : n_rows)) : 0;
+  };
+  int k0[A], k1[A], cb[A][R];
+  auto take = [&](int rp) {             // the lane's atoms of a group: bounds and first columns
 #pragma unroll
-    for (int c = 0; c < K; ++c) acc[c] = 0;
-    int k = k0;
-    for (; k + 4 <= k1; k += 4) {
-      int cb[4];
-      TL v[4][4];
+    for (int u = 0; u < A; ++u) {
+      k0[u] = __shfl_sync(0xffffffffu, rp, place * A + u) + slot;
+      k1[u] = __shfl_sync(0xffffffffu, rp, place * A + u + 1);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) cb[u] = __ldg(col + k + u);
+      for (int h = 0; h < R; ++h) cb[u][h] = k0[u] + SLOTS * h < k1[u] ? __ldg(col + k0[u] + SLOTS * h) : -1;
+    }
+  };
+  int rp = pointer(g), next = pointer(g + nw);
+  take(rp);
+  for (; g < groups; g += nw) {
+    TX s[4] = {0, 0, 0, 0};
+    for (bool first = true;; first = false) {
+      TL v[A][R][4];
+      int c[A][R];
+      bool more = false;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) RowVals<TV>::load(val, k + u, i, v[u]);
+      for (int u = 0; u < A; ++u) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        TX xv[4][K];
-        load_x<TX, K>(x, cb[u], xv);
+        for (int h = 0; h < R; ++h) {
+          c[u][h] = cb[u][h];
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-          for (int c = 0; c < K; ++c) acc[c] = fma((TX)v[u][jj], xv[jj][c], acc[c]);
+          for (int jj = 0; jj < 4; ++jj) v[u][h][jj] = 0;
+          if (c[u][h] >= 0) RowVals<TV>::load(val, k0[u] + SLOTS * h, i, v[u][h]);
+        }
+        more = more || k0[u] + SLOTS * R < k1[u];
       }
+      const bool again = __any_sync(0xffffffffu, more);
+      if (again) {
+#pragma unroll
+        for (int u = 0; u < A; ++u) {
+          k0[u] = min(k0[u] + SLOTS * R, k1[u]);
+#pragma unroll
+          for (int h = 0; h < R; ++h) cb[u][h] = k0[u] + SLOTS * h < k1[u] ? __ldg(col + k0[u] + SLOTS * h) : -1;
+        }
+      } else {
+        take(next);
+        next = pointer(g + 2 * nw);
+      }
+      TX xs[A][R][4][K];                // FP32: all x rows in flight too; FP64 has not the registers, nor the need
+      if constexpr (kAhead) {
+#pragma unroll
+        for (int u = 0; u < A; ++u)
+#pragma unroll
+          for (int h = 0; h < R; ++h) {
+#pragma unroll
+            for (int e = 0; e < 4 * K; ++e) xs[u][h][e / K][e % K] = 0;
+            if (c[u][h] >= 0) load_x<TX, K>(x, c[u][h], xs[u][h]);
+          }
+      }
+#pragma unroll
+      for (int u = 0; u < A; ++u)
+#pragma unroll
+        for (int h = 0; h < R; ++h) {
+          TX (&xv)[4][K] = xs[u][h];
+          if constexpr (!kAhead) {
+            if (c[u][h] < 0) continue;
+            load_x<TX, K>(x, c[u][h], xv);
+          }
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) {
+            TX w;
+            if constexpr (sizeof(TX) > sizeof(TL)) w = widen(v[u][h][jj]);
+            else w = (TX)v[u][h][jj];
+#pragma unroll
+            for (int q = 0; q < K; ++q) s[u * K + q] = fma(w, xv[jj][q], s[u * K + q]);
+          }
+        }
+      if (!again) break;
     }
-    for (; k < k1; ++k) {
-      TL v[4];
-      RowVals<TV>::load(val, k, i, v);
-      TX xv[4][K];
-      load_x<TX, K>(x, __ldg(col + k), xv);
+    TX t[2];
+    if constexpr (SLOTS == 8) {
+      const int hi = lane >> 4 & 1, lo = lane >> 3 & 1;
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj)
+      for (int q = 0; q < 2; ++q) t[q] = (hi ? s[2 + q] : s[q]) + __shfl_xor_sync(0xffffffffu, hi ? s[q] : s[2 + q], 16);
+      TX r = (lo ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, lo ? t[0] : t[1], 8);
+      r += __shfl_xor_sync(0xffffffffu, r, 4);
+      const int e = 2 * hi + lo;                  // atom e / K of the group, vector e % K
+      const int64_t a = g * PER + e / K;
+      if ((slot & 1) == 0 && a < n_rows) y[(4 * a + i) * K + e % K] = r;
+    } else {
+      const int hi = lane >> 3 & 1, lo = lane >> 2 & 1;
 #pragma unroll
-        for (int c = 0; c < K; ++c) acc[c] = fma((TX)v[jj], xv[jj][c], acc[c]);
+      for (int q = 0; q < 2; ++q) t[q] = (hi ? s[2 + q] : s[q]) + __shfl_xor_sync(0xffffffffu, hi ? s[q] : s[2 + q], 8);
+      const TX r = (lo ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, lo ? t[0] : t[1], 4);
+      const int e = 2 * hi + lo;
+      const int64_t a = g * PER + place * A + e / K;
+      if (a < n_rows) y[(4 * a + i) * K + e % K] = r;
     }
-    TX* yo = y + (4 * a + i) * K;
-#pragma unroll
-    for (int c = 0; c < K; ++c) yo[c] = acc[c];
   }
+}
+
+template <typename TV, typename TX, int K, int SLOTS>
+void spmv_launch(const mka_system* s, const TV* val, const TX* x, TX* y, int sms, cudaStream_t st) {
+  const int64_t per = (int64_t)(4 / K) * (8 / SLOTS) * (kSpmvThreads / 32);
+  const int64_t blocks = std::min<int64_t>((s->n_atoms + per - 1) / per, (int64_t)sms * kSpmvBlocks<TX, K>);
+  spmv_kernel<TV, TX, K, SLOTS><<<(unsigned)std::max<int64_t>(1, blocks), kSpmvThreads, 0, st>>>(
+      s->d_row_ptr, s->d_col, val, x, y, s->n_atoms);
 }
 
 template <typename TV, typename TX>
@@ -372,12 +458,15 @@ mka_status spmv_dispatch_k(const mka_system* s, const TV* val, const void* x, vo
   int dev = 0, sms = 0;
   MKA_CUDA_TRY(cudaGetDevice(&dev));
   MKA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((4 * s->n_atoms + 255) / 256, (int64_t)sms * 8));
   const TX* xx = reinterpret_cast<const TX*>(x);
   TX* yy = reinterpret_cast<TX*>(y);
-  if (k == 1) spmv_kernel<TV, TX, 1><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
-  else if (k == 2) spmv_kernel<TV, TX, 2><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
-  else spmv_kernel<TV, TX, 4><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
+  // Four slots waste less on rows of 13 blocks and add less (FP64, K = 4, 262,144 atoms: 492 against 539 us); eight spread
+  // a small system over more warps (512 atoms, K = 4: 8.8 against 10.9 us; 4,096 atoms, K = 1: 12.9 against 15). They meet at
+  // about eight warps an SM.
+  const bool wide = s->n_atoms * k < (int64_t)sms * 64;
+  if (k == 1) wide ? spmv_launch<TV, TX, 1, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 1, 4>(s, val, xx, yy, sms, st);
+  else if (k == 2) wide ? spmv_launch<TV, TX, 2, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 2, 4>(s, val, xx, yy, sms, st);
+  else wide ? spmv_launch<TV, TX, 4, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 4, 4>(s, val, xx, yy, sms, st);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
