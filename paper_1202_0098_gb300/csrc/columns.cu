@@ -1123,6 +1123,8 @@ mka_status allow_shared(const void* kernel, size_t* most) {
 // The general kernel's launch shape and, where they apply, the short recurrences': subspaces up to
 // kChainsMaxNu in reading A (beyond, the recurrences lose orthogonality on most atoms: at nu = 64 overlaps of
 // 1e-2 on 87-atom clusters), and the inner CG alone at any size.
+// A CTA per column (single.cu) where the subspace is well inside the clusters' space: where it nearly fills that, the
+// rounding of the sums decides at which vector a basis ends, and that stays with one kernel.
 mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl, int threads, int ctas_per_sm,
                         AtomsConfig* out) {
   const bool mixed = sh.arith != MKA_FP64;
@@ -1132,6 +1134,8 @@ mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl,
 #undef MKA_CFG
   const bool fits = nu <= kChainsMaxNu && 4 * (int64_t)max_cl >= 6 * nu;
   if (!s && !sh.general_only && (sh.cg_only || (!sh.mode_b && fits))) s = chains_config(sys, nu, sh.arith, ctas_per_sm, out);
+  if (!s && !mixed && !sh.general_only && !sh.cg_only && !sh.mode_b && max_cl >= nu && threads == 256)
+    s = single_config(sys, nu, out);
   return s;
 }
 
@@ -1143,6 +1147,9 @@ mka_status reduced_for(const mka_system* sys, const AtomsLaunchArgs& a, cudaStre
 mka_status atoms_launch(const mka_system* sys, int arith, const AtomsConfig& cf, const AtomsLaunchArgs& a,
                         cudaStream_t st) {
   const bool mixed = arith != MKA_FP64;
+  // few atoms: a CTA per column, from x0 = 0 and without keeping s_j
+  if (a.n_sel <= cf.single_max && !a.cg_only && !a.mode_b && !a.x0 && !a.prev_s && !a.keep_s && !a.fallback && a.grid <= 0)
+    return single_launch(sys, cf, a, st);
   if (cf.chains) {
     const mka_status s = chains_launch(sys, arith, cf, a, st);
     if (s || a.cg_only) return s;

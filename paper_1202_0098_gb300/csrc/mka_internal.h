@@ -103,6 +103,7 @@ struct AtomsConfig {
   int chains_grid = 0;     // its SMs x resident CTAs, dynamic shared memory and work slot
   size_t chains_smem = 0;
   size_t chains_slot = 0;
+  int single_max = 0;      // selections up to this many atoms run a CTA per column (0: none do)
 };
 // Subspaces up to this size run the short-recurrence kernel (chains.cu).
 constexpr int kChainsMaxNu = 48;
@@ -189,6 +190,9 @@ mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl,
 mka_status chains_config(const mka_system* sys, int nu, int arith, int ctas_per_sm, AtomsConfig* cf);
 mka_status chains_launch(const mka_system* sys, int arith, const AtomsConfig& cf, const AtomsLaunchArgs& a,
                          cudaStream_t st);
+// A CTA per column (single.cu; FP64, reading A): sets cf->single_max, and its launch, on the general kernel's slots.
+mka_status single_config(const mka_system* sys, int nu, AtomsConfig* cf);
+mka_status single_launch(const mka_system* sys, const AtomsConfig& cf, const AtomsLaunchArgs& a, cudaStream_t st);
 // Bytes of work slots the kernels need for selections of up to n atoms.
 inline size_t atoms_scratch_bytes(const AtomsConfig& cf, int64_t n) {
   const size_t g = cf.slot_bytes * (size_t)std::min<int64_t>(n, cf.grid_max);
