@@ -27,9 +27,7 @@ mka_status copy_selection(const mka_system* sys, const int64_t* atoms, int64_t n
 
 }  // namespace
 
-extern "C" {
-
-mka_status mka_cluster_sizes(const mka_system* sys, const int64_t* atoms, int64_t n_sel, int32_t* sizes) {
+mka_status mka::cluster_extents(const mka_system* sys, const int64_t* atoms, int64_t n_sel, int32_t* sizes, int32_t* rows) {
   if (!sys || !sizes) return fail(MKA_ERR_INVALID_ARG, "system and sizes are required");
   std::vector<int64_t> sel;
   mka_status s = copy_selection(sys, atoms, atoms ? n_sel : sys->n_atoms, sel);
@@ -38,16 +36,23 @@ mka_status mka_cluster_sizes(const mka_system* sys, const int64_t* atoms, int64_
   int64_t* d_sel = nullptr;
   int32_t* d_sizes = nullptr;
   MKA_CUDA_TRY(cudaMalloc(&d_sel, sizeof(int64_t) * n));
-  cudaError_t e = cudaMalloc(&d_sizes, sizeof(int32_t) * n);
+  cudaError_t e = cudaMalloc(&d_sizes, sizeof(int32_t) * n * (rows ? 2 : 1));
   if (e == cudaSuccess) e = cudaMemcpy(d_sel, sel.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    s = launch_cluster_sizes(sys, d_sel, n, d_sizes, sys->stream);
+    s = launch_cluster_sizes(sys, d_sel, n, d_sizes, rows ? d_sizes + n : nullptr, sys->stream);
     if (s == MKA_OK) e = cudaMemcpy(sizes, d_sizes, sizeof(int32_t) * n, cudaMemcpyDeviceToHost);
+    if (s == MKA_OK && e == cudaSuccess && rows) e = cudaMemcpy(rows, d_sizes + n, sizeof(int32_t) * n, cudaMemcpyDeviceToHost);
   }
   cudaFree(d_sel);
   cudaFree(d_sizes);
   if (e != cudaSuccess) return cuda_fail(e, "mka_cluster_sizes");
   return s;
+}
+
+extern "C" {
+
+mka_status mka_cluster_sizes(const mka_system* sys, const int64_t* atoms, int64_t n_sel, int32_t* sizes) {
+  return cluster_extents(sys, atoms, n_sel, sizes, nullptr);
 }
 
 void mka_result_destroy(mka_result* r) {
@@ -141,11 +146,11 @@ mka_status mka_solve_columns(mka_system* sys, const int64_t* atoms, int64_t n_se
   }
   // largest cluster of the selection sizes the per-CTA scratch
   int32_t* d_sizes = nullptr;
-  std::vector<int32_t> sizes(r->n_sel);
-  e = cudaMalloc(&d_sizes, sizeof(int32_t) * r->n_sel);
+  std::vector<int32_t> sizes(2 * r->n_sel);                 // and the blocks of their rows
+  e = cudaMalloc(&d_sizes, sizeof(int32_t) * 2 * r->n_sel);
   if (e == cudaSuccess) {
-    s = launch_cluster_sizes(sys, r->d_sel, r->n_sel, d_sizes, st);
-    if (s == MKA_OK) e = cudaMemcpyAsync(sizes.data(), d_sizes, sizeof(int32_t) * r->n_sel, cudaMemcpyDeviceToHost, st);
+    s = launch_cluster_sizes(sys, r->d_sel, r->n_sel, d_sizes, d_sizes + r->n_sel, st);
+    if (s == MKA_OK) e = cudaMemcpyAsync(sizes.data(), d_sizes, sizeof(int32_t) * 2 * r->n_sel, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
   cudaFree(d_sizes);
@@ -153,7 +158,8 @@ mka_status mka_solve_columns(mka_system* sys, const int64_t* atoms, int64_t n_se
     mka_result_destroy(r);
     return s != MKA_OK ? s : cuda_fail(e, "cluster sizes");
   }
-  const int max_cl = *std::max_element(sizes.begin(), sizes.end());
+  const int max_cl = *std::max_element(sizes.begin(), sizes.begin() + r->n_sel);
+  const int max_rows = *std::max_element(sizes.begin() + r->n_sel, sizes.end());
   if (prm->keep_s) {
     r->s_cap = std::max(1, std::min(max_cl, MKA_MAX_CLUSTER_ATOMS));
     e = cudaMalloc(&r->d_s_cl, sizeof(int32_t) * r->n_sel * r->s_cap);
@@ -163,7 +169,7 @@ mka_status mka_solve_columns(mka_system* sys, const int64_t* atoms, int64_t n_se
       return cuda_fail(e, "keep_s allocation");
     }
   }
-  s = launch_columns(sys, r, prm, max_cl, st);
+  s = launch_columns(sys, r, prm, max_cl, max_rows, st);
   if (s != MKA_OK) {
     mka_result_destroy(r);
     return s;
@@ -217,8 +223,8 @@ mka_status mka_cg_patch_targets(mka_system* sys, const int64_t* atoms, int64_t n
   std::vector<int64_t> sel(atoms, atoms + n);
   for (int64_t v : sel)
     if (v < 0 || v >= sys->n_atoms) return fail(MKA_ERR_INVALID_ARG, "atom index out of range");
-  std::vector<int32_t> sizes(n);
-  mka_status s = mka_cluster_sizes(sys, atoms, n, sizes.data());
+  std::vector<int32_t> sizes(n), rows(n);
+  mka_status s = cluster_extents(sys, atoms, n, sizes.data(), rows.data());
   if (s) return s;
   const int max_cl = *std::max_element(sizes.begin(), sizes.end());
   if (max_cl > MKA_MAX_CLUSTER_ATOMS) return fail(MKA_ERR_CLUSTER_TOO_LARGE, "cluster larger than the cap");
@@ -226,6 +232,7 @@ mka_status mka_cg_patch_targets(mka_system* sys, const int64_t* atoms, int64_t n
   AtomsShape sh;                                             // basis unused: smallest subspace
   sh.arith = arith;
   sh.cg_only = 1;
+  sh.max_rows = *std::max_element(rows.begin(), rows.end());
   s = atoms_config(sys, sh, max_cl, 256, 0, &cf);
   if (s) return s;
   cudaStream_t st = (cudaStream_t)stream;

@@ -646,9 +646,9 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
   const int nu = A.nu, m_cap = A.mcap;
   int* cl = reinterpret_cast<int*>(smem_raw);
   int* lrow = cl + A.clcap;
-  int* rbase = lrow + A.clcap + 1;
-  uint32_t* ent = reinterpret_cast<uint32_t*>(rbase + A.clcap);
-  size_t off = (size_t)(3 * A.clcap + 1 + A.lnnz_cap) * sizeof(int);
+  int* rbase = lrow + A.mcap / 4 + 1;
+  uint32_t* ent = reinterpret_cast<uint32_t*>(rbase + A.mcap / 4);
+  size_t off = (size_t)(A.clcap + 2 * (A.mcap / 4) + 1 + A.lnnz_cap) * sizeof(int);
   off = (off + 63) & ~(size_t)63;
   const int m4 = m_cap * 4;
   T* X0 = reinterpret_cast<T*>(smem_raw + off);
@@ -1378,7 +1378,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
 }
 
 size_t chains_smem_bytes(int clcap, int lnnz_cap, int mcap, size_t elem) {
-  const size_t off = (size_t)(3 * clcap + 1 + lnnz_cap) * sizeof(int);
+  const size_t off = (size_t)(clcap + 2 * (mcap / 4) + 1 + lnnz_cap) * sizeof(int);
   return align_up(off, 64) + (size_t)mcap * 4 * (elem == 4 ? 3 * sizeof(float) : 2 * sizeof(double));
 }
 

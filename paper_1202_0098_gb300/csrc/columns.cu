@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(NT, atoms_min_blocks<T, NT>()) atoms_kernel(co
       st.flag = lrow[ncl] <= A.lnnz_cap;
     }
     __syncthreads();
-    if (!st.flag) {  // cannot happen with a capacity of (largest cluster) x (longest row)
+    if (!st.flag) {  // cannot happen with a capacity of the most blocks of a cluster's rows
       for (int c = threadIdx.x; c < 4; c += blockDim.x) {
         A.status[4 * widx + c] = ST_TOOLARGE;
         A.nu_eff[4 * widx + c] = 0;
@@ -994,8 +994,8 @@ __global__ void __launch_bounds__(NT, atoms_min_blocks<T, NT>()) atoms_kernel(co
   }
 }
 
-// One warp per atom: cluster size only.
-__global__ void cluster_size_kernel(Args<double> A, int32_t* sizes) {
+// One warp per atom: the cluster's size and (rows not NULL) the blocks of its atoms' rows, which bound its local blocks.
+__global__ void cluster_size_kernel(Args<double> A, int32_t* sizes, int32_t* rows) {
   const int lane = threadIdx.x & 31;
   const int64_t wglobal = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -1007,16 +1007,24 @@ __global__ void cluster_size_kernel(Args<double> A, int32_t* sizes) {
     const int nx = cell_range(cell_coord(px, A.cell_len[0], A.ncell[0]), A.ncell[0], rx);
     const int ny = cell_range(cell_coord(py, A.cell_len[1], A.ncell[1]), A.ncell[1], ry);
     const int nz = cell_range(cell_coord(pz, A.cell_len[2], A.ncell[2]), A.ncell[2], rz);
-    int count = 0;
+    int count = 0, blocks = 0;
     for (int ci = 0; ci < nx * ny * nz; ++ci) {
       const int ix = ci / (ny * nz), iy = (ci / nz) % ny, iz = ci % nz;
       const int c = (rx[ix] * A.ncell[1] + ry[iy]) * A.ncell[2] + rz[iz];
       for (int k = A.cell_start[c] + lane; k < A.cell_start[c + 1]; k += 32)
-        count += within_R(A.pos, A.posf, A.box, A.R2, A.pre_lo, A.pre_hi, A.cell_atoms[k], px, py, pz, pxf, pyf,
-                          pzf);
+      {
+        const int b = A.cell_atoms[k];
+        if (!within_R(A.pos, A.posf, A.box, A.R2, A.pre_lo, A.pre_hi, b, px, py, pz, pxf, pyf, pzf)) continue;
+        ++count;
+        if (rows) blocks += A.row_ptr[b + 1] - A.row_ptr[b];
+      }
     }
     count = warp_sum(count);
-    if (lane == 0) sizes[i] = count;
+    if (rows) blocks = warp_sum(blocks);
+    if (lane == 0) {
+      sizes[i] = count;
+      if (rows) rows[i] = blocks;
+    }
   }
 }
 
@@ -1043,7 +1051,7 @@ size_t slot_bytes_for(int nu, int mcap, size_t elem) {
 }
 
 template <typename TV, typename T, int NT>
-mka_status config_t(const mka_system* sys, int nu, int max_cl, int ctas_per_sm, AtomsConfig* out) {
+mka_status config_t(const mka_system* sys, int nu, int max_cl, int max_rows, int ctas_per_sm, AtomsConfig* out) {
   AtomsConfig cf{};
   cf.threads = NT;
   if (sys->max_row_blocks > 255)
@@ -1051,6 +1059,9 @@ mka_status config_t(const mka_system* sys, int nu, int max_cl, int ctas_per_sm, 
   const int cl_atoms = std::max(1, std::min(max_cl, kMaxCl));
   cf.mcap = 4 * cl_atoms;
   cf.lnnz_cap = cl_atoms * std::max(1, sys->max_row_blocks);
+  // the rows' own blocks are a tighter bound: 250-atom clusters of rows of 8 to 22 blocks, FP32, 82 -> 71 KB, three CTAs an
+  // SM instead of two (the short recurrences' kernel at nu = 40, 2,501 atoms: 30 -> 26 ms)
+  if (max_rows > 0) cf.lnnz_cap = std::min(cf.lnnz_cap, max_rows);
   cf.clcap = 2;
   while (cf.clcap < cl_atoms) cf.clcap <<= 1;
   cf.smem = dyn_smem_bytes(nu, cf.clcap, cf.lnnz_cap, cf.mcap, sizeof(T));
@@ -1090,7 +1101,7 @@ mka_status launch_t(const mka_system* sys, const AtomsConfig& cf, const AtomsLau
 }  // namespace
 
 mka_status launch_cluster_sizes(const mka_system* sys, const int64_t* d_sel, int64_t n_sel, int32_t* d_sizes,
-                                cudaStream_t st) {
+                                int32_t* d_rows, cudaStream_t st) {
   Args<double> A{};
   fill_system_args(A, sys);
   A.sel = d_sel;
@@ -1100,7 +1111,7 @@ mka_status launch_cluster_sizes(const mka_system* sys, const int64_t* d_sel, int
   MKA_CUDA_TRY(cudaGetDevice(&dev));
   MKA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t blocks = std::min<int64_t>((n_sel + 7) / 8, (int64_t)sms * 16);
-  cluster_size_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), threads, 0, st>>>(A, d_sizes);
+  cluster_size_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), threads, 0, st>>>(A, d_sizes, d_rows);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
@@ -1129,7 +1140,7 @@ mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl,
                         AtomsConfig* out) {
   const bool mixed = sh.arith != MKA_FP64;
   const int nu = sh.p + sh.q;
-#define MKA_CFG(TV, T, NT) config_t<TV, T, NT>(sys, nu, max_cl, ctas_per_sm, out)
+#define MKA_CFG(TV, T, NT) config_t<TV, T, NT>(sys, nu, max_cl, sh.max_rows, ctas_per_sm, out)
   mka_status s = MKA_DISPATCH(MKA_CFG, sys->storage, mixed, threads);
 #undef MKA_CFG
   const bool fits = nu <= kChainsMaxNu && 4 * (int64_t)max_cl >= 6 * nu;
@@ -1159,7 +1170,7 @@ mka_status atoms_launch(const mka_system* sys, int arith, const AtomsConfig& cf,
 #undef MKA_LAUNCH
 }
 
-mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_params* prm, int max_cl,
+mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_params* prm, int max_cl, int max_rows,
                           cudaStream_t st) {
   const int nu = prm->p + prm->q;
   AtomsConfig cf{};
@@ -1168,6 +1179,7 @@ mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_para
   sh.q = prm->q;
   sh.arith = prm->arith;
   sh.mode_b = prm->subspace == MKA_SUBSPACE_B;
+  sh.max_rows = max_rows;
   mka_status s = atoms_config(sys, sh, max_cl, 256, 0, &cf);
   if (s) return s;
   // atoms per chunk: the reduced-problem buffer of a chunk stays within 2 GiB

@@ -53,6 +53,7 @@ struct mka_system {
   mka_sk_params sk{};           // the model's Slater-Koster parameters (forces need their derivatives)
   bool have_sk = false;         // false for a caller's BSR matrices: no forces
   int max_cluster = -1;         // largest cluster over all atoms (-1: not computed yet)
+  int max_cluster_rows = 0;     // and the most blocks in the rows of one cluster's atoms
   mka::CellList cells{};
   // host copies of the pattern
   std::vector<int32_t> h_row_ptr, h_col;
@@ -182,6 +183,7 @@ struct AtomsShape {
   int mode_b = 0;          // reading B: the general kernel only
   int cg_only = 0;         // the inner CG only
   int general_only = 0;    // no leftover list at hand: the general kernel only
+  int max_rows = 0;        // most blocks in the rows of one cluster's atoms (0: not known)
 };
 mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl, int threads, int ctas_per_sm,
                         AtomsConfig* out);
@@ -208,9 +210,11 @@ mka_status atoms_launch(const mka_system* sys, int arith, const AtomsConfig& cf,
 
 // Kernels launched from the C entry points (defined in the .cu files).
 mka_status launch_cluster_sizes(const mka_system* sys, const int64_t* d_sel, int64_t n_sel, int32_t* d_sizes,
-                                cudaStream_t st);
+                                int32_t* d_rows, cudaStream_t st);
+// mka_cluster_sizes with the blocks of each cluster's rows (rows: [n_sel] or NULL).
+mka_status cluster_extents(const mka_system* sys, const int64_t* atoms, int64_t n_sel, int32_t* sizes, int32_t* rows);
 mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_params* prm, int max_cluster_atoms,
-                          cudaStream_t st);
+                          int max_rows, cudaStream_t st);
 mka_status launch_find_mu(mka_result* res, double n_electrons, double kT, double tol, double* mu_out);
 mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT, double* rho_out,
                           double* e_band, double* n_elec);

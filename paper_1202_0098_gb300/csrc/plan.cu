@@ -159,7 +159,7 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   MKA_CUDA_TRY(cudaMemsetAsync(P->counter, 0, sizeof(int) * kAtomsCounters, st));
   const int32_t* order = nullptr;
   if (P->tune.order_by_size) {
-    mka_status s = launch_cluster_sizes(P->sys, r->d_sel, n, P->sizes, st);
+    mka_status s = launch_cluster_sizes(P->sys, r->d_sel, n, P->sizes, nullptr, st);
     if (s) return s;
     MKA_CUDA_TRY(cudaMemsetAsync(P->bins, 0, sizeof(int32_t) * kSizeBins, st));
     const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 1024);
@@ -279,12 +279,13 @@ mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_p
   P->max_atoms = max_atoms;
   // largest cluster of the whole system sizes every work slot (computed once per system)
   if (sys->max_cluster < 0) {
-    std::vector<int32_t> sz(sys->n_atoms);
-    mka_status s0 = mka_cluster_sizes(sys, nullptr, sys->n_atoms, sz.data());
+    std::vector<int32_t> sz(sys->n_atoms), rows(sys->n_atoms);
+    mka_status s0 = cluster_extents(sys, nullptr, sys->n_atoms, sz.data(), rows.data());
     if (s0) {
       delete P;
       return s0;
     }
+    sys->max_cluster_rows = *std::max_element(rows.begin(), rows.end());
     sys->max_cluster = *std::max_element(sz.begin(), sz.end());
   }
   mka_status s = MKA_OK;
@@ -298,6 +299,7 @@ mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_p
   sh.q = prm->q;
   sh.arith = prm->arith;
   sh.mode_b = prm->subspace == MKA_SUBSPACE_B;
+  sh.max_rows = sys->max_cluster_rows;
   s = atoms_config(sys, sh, P->max_cl, t.threads, t.ctas_per_sm, &P->cf);
   if (s) {
     delete P;
