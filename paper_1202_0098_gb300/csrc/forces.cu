@@ -63,10 +63,10 @@ struct ForceBlockArgs {
 constexpr int kForceThreads = 128, kForceBlocks = 32;   // threads of a CTA; pattern blocks it takes at a time
 
 __global__ void __launch_bounds__(kForceThreads) force_blocks_kernel(const ForceBlockArgs A) {
-  extern __shared__ __align__(16) double sm[];    // g = C diag(x) V_j and x for x = f, f eps: 8 nu each; rho, pi
+  extern __shared__ __align__(16) double sm[];    // g = C diag(x) V_j for x = f, f eps: 8 nu; x, then rho and pi over it
   const int nu = A.nu;
   double *gv = sm, *f = sm + 8 * nu, *fe = f + 4 * nu;
-  double *s_rho = sm + 16 * nu, *s_pi = s_rho + 17 * kForceBlocks;
+  double *s_rho = f, *s_pi = s_rho + 17 * kForceBlocks;
   const int64_t t = blockIdx.x;
   const int64_t atom = A.sel[t];
   const int64_t k0 = A.row_ptr[atom];
@@ -178,7 +178,7 @@ mka_status force_blocks_enqueue(const mka_system* sys, const int64_t* sel, const
   A.out_base = out_base;
   A.pi = pi;
   A.g = g;
-  force_blocks_kernel<<<(unsigned)n_sel, kForceThreads, sizeof(double) * (16 * nu + 2 * 17 * kForceBlocks), st>>>(A);
+  force_blocks_kernel<<<(unsigned)n_sel, kForceThreads, sizeof(double) * (8 * nu + std::max(8 * nu, 2 * 17 * kForceBlocks)), st>>>(A);
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
