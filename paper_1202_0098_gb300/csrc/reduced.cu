@@ -444,13 +444,37 @@ __device__ __forceinline__ double team_sum(double v) {
 // Doubles of shared memory per column: two packed triangles and three vectors.
 __host__ __device__ constexpr int team_doubles(int n) { return n * (n + 1) + 3 * n; }
 
+// TL lanes a column; a team of more than a warp has a CTA to itself: above nu = 64, where few columns fit on an SM and a
+// warp's FP64 instructions, one in 64 cycles, are what a column waits for (148 columns of nu = 100: 6.6 -> 3.2 ms).
+template <int TL>
+__device__ __forceinline__ void team_sync() {
+  if constexpr (TL > 32) __syncthreads();
+  else __syncwarp();
+}
+
 template <int TL, int NS>
-__global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
-  constexpr int CPW = 32 / TL;
+__global__ void __launch_bounds__(TL > 32 ? TL : 32) team_tridiag_kernel(const RedArgs A) {
+  constexpr int CPW = TL > 32 ? 1 : 32 / TL;
   extern __shared__ double sm[];
+  __shared__ double share[1 + 2 * (TL > 32 ? TL / 32 : 1)];   // across a team's warps: a pivot, two sums
   const int lane = threadIdx.x, c = lane % CPW, l = lane / CPW, nu = A.nu;
   const int64_t col = (int64_t)blockIdx.x * CPW + c;
   const bool real = col < A.n_cols;
+  const int wl = TL > 32 ? l & ~31 : 0, ww_ = TL > 32 ? 32 : TL;   // the lanes of this warp within the team
+  // sum over the team; `at` keeps neighbouring sums apart
+  auto sum = [&](double v, int at) {
+    if constexpr (TL > 32) {
+      v = team_sum<1>(v);
+      if ((l & 31) == 0) share[1 + at * (TL / 32) + (l >> 5)] = v;
+      __syncthreads();
+      v = 0.0;
+#pragma unroll
+      for (int w = 0; w < TL / 32; ++w) v += share[1 + at * (TL / 32) + w];
+      return v;
+    } else {
+      return team_sum<CPW>(v);
+    }
+  };
   const int64_t colr = real ? col : A.n_cols - 1;
   const Lane M{A.blk + (size_t)(colr >> 5) * red_block_doubles(nu) * 32 + (colr & 31), nu};
   const Scratch Z = scratch_of(M);
@@ -469,7 +493,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       L[pk(i, j) * CPW] = in ? M.S(i, j) : (i == j ? 1.0 : 0.0);
       H[pk(i, j) * CPW] = in ? M.H(j, i) : 0.0;
     }
-  __syncwarp();
+  team_sync<TL>();
   // Cholesky, a column at a time from the ones before
   bool spd = true;
   for (int k = 0; k < nm; ++k) {
@@ -483,19 +507,25 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       const double lk = L[pk(k, j) * CPW];
 #pragma unroll
       for (int s = 0; s < NS; ++s)
-        if (TL * (s + 1) > k && TL * s < nm) v[s] = fma(-(l + TL * s < nm ? L[pk(l + TL * s, j) * CPW] : 0.0), lk, v[s]);
+        if (wl + ww_ + TL * s > k && wl + TL * s < nm) v[s] = fma(-(l + TL * s < nm ? L[pk(l + TL * s, j) * CPW] : 0.0), lk, v[s]);
     }
     double dk = 0.0;
 #pragma unroll
     for (int s = 0; s < NS; ++s)
       if (s == k / TL) dk = v[s];
-    dk = __shfl_sync(0xffffffffu, dk, (k % TL) * CPW + c);
+    if constexpr (TL > 32) {
+      if (l == k % TL) share[0] = dk;
+      __syncthreads();
+      dk = share[0];
+    } else {
+      dk = __shfl_sync(0xffffffffu, dk, (k % TL) * CPW + c);
+    }
     if (!(dk > 0.0)) {
       spd = false;
       dk = 1.0;
     }
     const double lkk = sqrt(dk), r = 1.0 / lkk;
-    __syncwarp();
+    team_sync<TL>();
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       const int i = l + TL * s;
@@ -505,7 +535,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
         rd[k * CPW] = r;
       }
     }
-    __syncwarp();
+    team_sync<TL>();
   }
   // X = L^{-1} H, upper triangle: row i of the packed lower triangle is column i of X, a lane's own
   for (int j = 0; j < nm; ++j) {
@@ -519,7 +549,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       const double lk = L[pk(j, k) * CPW];
 #pragma unroll
       for (int s = 0; s < NS; ++s)
-        if (TL * (s + 1) > j && TL * s < nm) v[s] = fma(-(l + TL * s < nm ? H[pk(l + TL * s, k) * CPW] : 0.0), lk, v[s]);
+        if (wl + ww_ + TL * s > j && wl + TL * s < nm) v[s] = fma(-(l + TL * s < nm ? H[pk(l + TL * s, k) * CPW] : 0.0), lk, v[s]);
     }
     const double r = rd[j * CPW];
 #pragma unroll
@@ -528,7 +558,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       if (i >= j && i < nm) H[pk(i, j) * CPW] = v[s] * r;
     }
   }
-  __syncwarp();
+  team_sync<TL>();
   // A = L^{-1} X^T, lower triangle, column by column: the known part A(j, k), k < j, then the substitution
   for (int j = 0; j < nm; ++j) {
     double v[NS];
@@ -541,17 +571,17 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       const double a = H[pk(j, k) * CPW];
 #pragma unroll
       for (int s = 0; s < NS; ++s)
-        if (TL * (s + 1) > j && TL * s < nm) v[s] = fma(-(l + TL * s < nm ? L[pk(l + TL * s, k) * CPW] : 0.0), a, v[s]);
+        if (wl + ww_ + TL * s > j && wl + TL * s < nm) v[s] = fma(-(l + TL * s < nm ? L[pk(l + TL * s, k) * CPW] : 0.0), a, v[s]);
     }
     for (int k = j; k < nm; ++k) {
 #pragma unroll
       for (int s = 0; s < NS; ++s)
         if (l + TL * s == k) H[pk(k, j) * CPW] = v[s] * rd[k * CPW];
-      __syncwarp();
+      team_sync<TL>();
       const double a = H[pk(k, j) * CPW];
 #pragma unroll
       for (int s = 0; s < NS; ++s)
-        if (TL * (s + 1) > k && TL * s < nm)
+        if (wl + ww_ + TL * s > k && wl + TL * s < nm)
           v[s] = fma(-(l + TL * s > k && l + TL * s < nm ? L[pk(l + TL * s, k) * CPW] : 0.0), a, v[s]);
     }
   }
@@ -565,14 +595,14 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       v[s] = on && i > k && i < nm ? H[pk(i, k) * CPW] : 0.0;
       s2 = fma(v[s], v[s], s2);
     }
-    s2 = team_sum<CPW>(s2);
+    s2 = sum(s2, 0);
     const double x0 = on ? H[pk(k + 1, k) * CPW] : 0.0;
     const double nrm = sqrt(s2);
     const double alpha = x0 >= 0.0 ? -nrm : nrm;
     const double v0 = x0 - alpha;
     const double vtv = s2 - x0 * x0 + v0 * v0;
     const double tk = vtv > 0.0 ? 2.0 / vtv : 0.0;          // H_k = I - tk v v^T
-    __syncwarp();
+    team_sync<TL>();
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       const int i = l + TL * s;
@@ -587,7 +617,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       Z.e(k) = alpha;
       Z.tau(k) = tk;
     }
-    __syncwarp();
+    team_sync<TL>();
     double p[NS], pv = 0.0;
 #pragma unroll
     for (int s = 0; s < NS; ++s) p[s] = 0.0;
@@ -596,7 +626,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       const int jr = pk(j, 0);
 #pragma unroll
       for (int s = 0; s < NS; ++s)
-        if (TL * (s + 1) > k + 1 && TL * s < nm) {
+        if (wl + ww_ + TL * s > k + 1 && wl + TL * s < nm) {
           const int i = l + TL * s;
           const int o = j <= i ? pk(i, j) : jr + i;
           p[s] = fma(i > k && i < nm ? H[o * CPW] : 0.0, vj, p[s]);
@@ -607,14 +637,14 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
       p[s] *= tk;
       pv = fma(p[s], v[s], pv);
     }
-    pv = team_sum<CPW>(pv);
+    pv = sum(pv, 1);
     const double kc = 0.5 * tk * pv;
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       p[s] = fma(-kc, v[s], p[s]);                           // w = p - kc v
       if (l + TL * s < nm) ww[(l + TL * s) * CPW] = p[s];
     }
-    __syncwarp();
+    team_sync<TL>();
     for (int j = k + 1; j < nm; ++j) {                       // B -= v w^T + w v^T
       const double vj = vv[j * CPW], wj = ww[j * CPW];
 #pragma unroll
@@ -626,7 +656,7 @@ __global__ void __launch_bounds__(32) team_tridiag_kernel(const RedArgs A) {
         }
       }
     }
-    __syncwarp();
+    team_sync<TL>();
   }
   if (!real) return;
   if (l == 0) {
@@ -932,14 +962,14 @@ __global__ void __launch_bounds__(32) team_vectors_kernel(const RedArgs A) {
 //   one lane per column once there are enough of them to fill the chip that way, it has no idle lanes (524,288
 //   columns of nu = 30: 158, 0.30 us a column against the teams' 0.44): from about 40,000 columns up to nu = 32, and
 //   16,000 up to nu = 64, where a lane's rate is 0.7 us and a team's 1.5;
-//   nu up to 160 (the packed triangles fit in shared memory): a warp per column at any count (148 columns of nu = 100:
-//   52 against 445); below nu = 5 the scratch between the three kernels does not fit.
+//   nu up to 160 (the packed triangles fit in shared memory): four warps, then a warp per column at any count (148 columns
+//   of nu = 100: 9 against 445); below nu = 5 the scratch between the three kernels does not fit.
 constexpr int64_t kFewColumns = 2048, kManyColumns32 = 40960, kManyColumns64 = 16384;
 
 // TL1 lanes a column in the first kernel, TL2 in the last; nu <= TL NS.
 template <int TL1, int NS1, int TL2, int NS2>
 mka_status team_launch(const RedArgs& A, cudaStream_t st) {
-  constexpr int C1 = 32 / TL1, C2 = 32 / TL2;
+  constexpr int C1 = TL1 > 32 ? 1 : 32 / TL1, C2 = 32 / TL2;
   auto k1 = team_tridiag_kernel<TL1, NS1>;
   auto k2 = team_vectors_kernel<TL2, NS2>;
   mka_status s = allow_shared(reinterpret_cast<const void*>(k1), nullptr);
@@ -948,7 +978,7 @@ mka_status team_launch(const RedArgs& A, cudaStream_t st) {
   if (!s) s = allow_shared(reinterpret_cast<const void*>(k2), nullptr);
   if (s) return s;
   const size_t smem = sizeof(double) * team_doubles(A.nu);
-  k1<<<(unsigned)((A.n_cols + C1 - 1) / C1), 32, smem * C1, st>>>(A);
+  k1<<<(unsigned)((A.n_cols + C1 - 1) / C1), TL1 > 32 ? TL1 : 32, smem * C1, st>>>(A);
   if (A.n_cols <= kFewColumns)
     bisect_kernel<<<(unsigned)(A.n_cols * ((A.nu + 31) / 32)), 32, sizeof(double) * 2 * A.nu, st>>>(A);
   else
@@ -975,7 +1005,7 @@ mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, 
   A.cv = cv;
   A.col0 = col0;
   if (nu >= kTeamMinNu && nu <= 160) {
-    if (nu > 64) return team_launch<32, 5, 32, 5>(A, st);
+    if (nu > 64) return team_launch<128, 2, 32, 5>(A, st);
     if (nu > 32) {
       if (n_cols <= kFewColumns) return team_launch<32, 2, 32, 2>(A, st);
       if (n_cols <= kManyColumns64) return team_launch<16, 4, 32, 2>(A, st);
