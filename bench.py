@@ -7,11 +7,11 @@ CG start. The timed region is the whole work flow of Eq. EQ-WORK-FLOW over the
 whole system: K steps, each one slice of N/K atoms solved by graph-replayed
 plan batches (cluster extraction, inner CG, multiple Krylov basis, projection,
 reduced eigensolve) whose levels and rho pieces a sweep keeps in HBM; after the
-last slice, one mu by bisection over all 4.03e7 columns, rho on the whole
+last slice, one mu over all 4.03e7 columns, rho on the whole
 pattern and the band energy at that mu. `value` = 4 N / (timed seconds).
 
 Under torchrun each rank sweeps one chunk-aligned range of the atoms; mu and
-the energies come from one all-reduce of chunk sums per bisection halving
+the energies come from one all-reduce of chunk sums per root-finder step
 (paper_1202_0098_gb300.distributed), bit-identical to one process.
 
 Also reported: K1 (the global BSR SpMV) in GB/s against the measured HBM peak,
@@ -501,7 +501,7 @@ def spmv_leg(mka, torch, sysh, stream, reps=20):
 
 
 def sample_window(mka, plan, atoms, w, half):
-    """mu of a random sample of atoms (the plan's batch bisection), and the sweep window around it:
+    """mu of a random sample of atoms (the plan's own mu), and the sweep window around it:
     [mu_s - half - 40 kT, mu_s + half + 40 kT]; the largest number of window levels in a sample column."""
     mka.mka_plan_run(plan, atoms, w.electrons_per_atom * len(atoms), w.kT, None)
     mu_s, _, _ = mka.mka_plan_scalars(plan)

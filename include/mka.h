@@ -13,7 +13,7 @@
  *   - solve the reduced nu x nu problem (Eq. EQ-SUB-EIG-VEC);
  *   - form the Fermi-weighted density matrix rho_ij (Eq. EQ-DM), the subspace
  *     Green's function G_ij(z) (Eq. EQ-SOLUTION-SUB-GZ) and the band energy
- *     (Eq. EQ-ENE); mu is found by bisection on the electron count (Sec. 2).
+ *     (Eq. EQ-ENE); mu is the root of the electron count (Sec. 2).
  * Every column works on the real-space projection of H and S onto the
  * cluster of atoms within a radius R of j's atom (Sec. 3).
  *
@@ -423,7 +423,7 @@ mka_status mka_autotune_batch(mka_system* sys, const mka_solve_params* prm, cons
 /* The work flow of Eq. EQ-WORK-FLOW over a whole system (or one contiguous range
  * of its atoms, for a process that owns that range): first every column's
  * levels (eps_alpha, w_alpha), then one chemical potential from the total
- * electron count of all of them (Sec. 2, bisection), then rho_ij (Eq. EQ-DM) and
+ * electron count of all of them (Sec. 2), then rho_ij (Eq. EQ-DM) and
  * the band energy (Eq. EQ-ENE) at that mu.
  *
  * A sweep keeps, in device memory, for every column of its range: the levels and

@@ -1,12 +1,12 @@
 // The per-atom solve with a CTA for each of the atom's four columns: FP64, for selections too small to fill the chip.
 //
 // The kernels that take an atom's four columns together read every block once for the four, which is the better way
-// where there are atoms enough: at FP64 an SM works off two lanes a cycle, and one atom's products, orthogonalisation and
-// projection are 36 ms of them at nu = 100 (640 rows) whatever the other 151 SMs do; 8.4 with a CTA a column. The columns of an atom are independent,
-// so up to a CTA per SM their four parts run side by side. The steps are the general kernel's (columns.cu) for one
-// column: CG for s_j, then one classical Gram-Schmidt pass with the Gram correction c - E c a vector and the projection of
-// the previous vector in the same sweep; the sums' order differs. A row is a thread's in all of them, 640 rows are five warps to
-// a scheduler, which keeps the FP64 pipe busy behind its own latency.
+// where there are atoms enough: at FP64 an SM works off two lanes a cycle, and one atom's products, orthogonalisation
+// and projection are 36 ms of them at nu = 100 (640 rows) whatever the other 151 SMs do; 8.4 with a CTA a column (1.6
+// against 4.8 at nu = 30). The columns of an atom are independent, so up to a CTA per SM their four parts run side by
+// side. The steps are the general kernel's (columns.cu) for one column: CG for s_j, then one classical Gram-Schmidt pass
+// with the Gram correction c - E c a vector, the previous vector's projection in the same sweep; the sums' order differs.
+// A row is a thread's in all of them: 640 rows are five warps to a scheduler, enough to hide the FP64 pipe's latency.
 #include "atoms.cuh"
 
 namespace mka {
