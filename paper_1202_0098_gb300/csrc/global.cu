@@ -445,6 +445,54 @@ __global__ void __launch_bounds__(kSpmvThreads, (kSpmvBlocks<TX, K>))
   }
 }
 
+// BF16 values with one or two FP32 vectors on large systems: a thread per row, four blocks in flight. A block is 32 bytes
+// there and a load by slots half as wide as the lanes could take, so that the instructions of the kernel above bound it, not
+// memory (262,144 / 5.8 million atoms: one vector 38 / 784 us by slots, 32 / 697 by rows; two 42 / 875 and 42 / 813; four
+// 68 / 1,466 and 73 / 1,550).
+template <int K>
+__global__ void __launch_bounds__(256) spmv_bf16_rows_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+                                                             const __nv_bfloat16* __restrict__ val,
+                                                             const float* __restrict__ x, float* __restrict__ y, int64_t n_rows) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < 4 * n_rows; g += stride) {
+    const int64_t a = g >> 2;
+    const int i = (int)(g & 3);
+    const int k0 = __ldg(row_ptr + a), k1 = __ldg(row_ptr + a + 1);
+    float acc[K];
+#pragma unroll
+    for (int c = 0; c < K; ++c) acc[c] = 0.0f;
+    int k = k0;
+    for (; k + 4 <= k1; k += 4) {
+      int cb[4];
+      float v[4][4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cb[u] = __ldg(col + k + u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) RowVals<__nv_bfloat16>::load(val, k + u, i, v[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float xv[4][K];
+        load_x<float, K>(x, cb[u], xv);
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+          for (int c = 0; c < K; ++c) acc[c] = fmaf(v[u][jj], xv[jj][c], acc[c]);
+      }
+    }
+    for (; k < k1; ++k) {
+      float v[4], xv[4][K];
+      RowVals<__nv_bfloat16>::load(val, k, i, v);
+      load_x<float, K>(x, __ldg(col + k), xv);
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+        for (int c = 0; c < K; ++c) acc[c] = fmaf(v[jj], xv[jj][c], acc[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < K; ++c) y[g * K + c] = acc[c];
+  }
+}
+
 template <typename TV, typename TX, int K, int SLOTS>
 void spmv_launch(const mka_system* s, const TV* val, const TX* x, TX* y, int sms, cudaStream_t st) {
   const int64_t per = (int64_t)(4 / K) * (8 / SLOTS) * (kSpmvThreads / 32);
@@ -460,6 +508,15 @@ mka_status spmv_dispatch_k(const mka_system* s, const TV* val, const void* x, vo
   MKA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const TX* xx = reinterpret_cast<const TX*>(x);
   TX* yy = reinterpret_cast<TX*>(y);
+  if constexpr (std::is_same<TV, __nv_bfloat16>::value && sizeof(TX) == 4)
+    if (k <= 2 && s->n_atoms >= (k == 1 ? 65536 : 131072)) {   // below, both take the same time or the slots less
+      const int64_t blocks = std::min<int64_t>((4 * s->n_atoms + 255) / 256, (int64_t)sms * 8);
+      if (k == 1) spmv_bf16_rows_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
+      else spmv_bf16_rows_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
+      count_launches();
+      MKA_CUDA_TRY(cudaGetLastError());
+      return MKA_OK;
+    }
   // Four slots waste less on rows of 13 blocks and add less (FP64, K = 4, 262,144 atoms: 492 against 539 us); eight spread
   // a small system over more warps (512 atoms, K = 4: 8.8 against 10.9 us; 4,096 atoms, K = 1: 12.9 against 15). They meet at
   // about eight warps an SM.

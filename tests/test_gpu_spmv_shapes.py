@@ -1,6 +1,6 @@
 """The global products at the edges of their kernels: systems below and above the change from eight to four slots, row
-counts that are no multiple of a warp's atoms, rows of 1 to about 55 blocks (more than a batch of 8 and of 16), all value
-and vector types. Against a row-by-row product of the stored values in FP64: sums of n products differ by at most
+counts that are no multiple of a warp's atoms, the change to rows for BF16 on large systems, rows of 1 to about 55 blocks
+(more than a batch of 8 and of 16), all value and vector types. Against a row-by-row product of the stored values in FP64: sums of n products differ by at most
 (n + 2) roundings of the vector's type times the sum of the magnitudes."""
 import numpy as np
 import pytest
@@ -11,9 +11,11 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("lattice,a,vac,cells", [("diamond", 3.567, 0.0, 4), ("fcc", 4.0, 0.55, 5), ("fcc", 2.3, 0.03, 5),
-                                                 ("diamond", 3.567, 0.01, 11)])
-@pytest.mark.parametrize("storage", ["fp64", "fp32", "bf16"])
+SMALL = [("diamond", 3.567, 0.0, 4), ("fcc", 4.0, 0.55, 5), ("fcc", 2.3, 0.03, 5), ("diamond", 3.567, 0.01, 11)]
+
+
+@pytest.mark.parametrize("lattice,a,vac,cells,storage", [(*c, t) for c in SMALL for t in ("fp64", "fp32", "bf16")] +
+                         [("diamond", 3.567, 0.01, 26, "bf16")])    # above 131,072 atoms: rows, not slots
 def test_products(lattice, a, vac, cells, storage):
     from paper_1202_0098_gb300 import build, mka
     build.build()
