@@ -179,16 +179,15 @@ def reduced_flops(nu):
 
 def column_flops(m, nnz, nu, cg_it, n_pattern_rows):
     """Algorithmic FLOPs of one column, counted as plain arithmetic: the products of the CG and
-    the basis, CG vector work, one Gram-Schmidt pass per vector (coefficients and update), norms,
-    the projection, the reduced solve and the rows V_j, (S V)_j of the outputs."""
+    the basis, CG vector work, the vector work of the short recurrences, the sums of S_r, the reduced
+    solve and the rows V_j, (S V)_j of the outputs."""
     spmv = 2.0 * 16.0 * nnz * (cg_it + 2 * nu)          # CG S-products + nu S- and nu H-products
     cg_vec = 10.0 * m * cg_it                            # two dots, three axpys per CG step
-    gs = 2.0 * m * nu * (nu - 1)                          # one pass of dots + updates per new vector
-    norms = 4.0 * m * nu                                  # S-norm and scaling per vector
-    proj = 4.0 * m * nu * nu                              # U^T K and U^T (S U)
+    rec = 20.0 * m * nu                                   # four dots and six axpys per vector
+    proj = 1.0 * m * nu * nu                              # S_r, one triangle
     red = reduced_flops(nu)                               # the reduced generalized eigensolve
     out = 4.0 * nu * nu                                   # V_j and (S V)_j
-    return spmv + cg_vec + gs + norms + proj + red + out
+    return spmv + cg_vec + rec + proj + red + out
 
 
 def oracle_pool(mp, cores):
@@ -807,13 +806,13 @@ def main():
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     mhz = clk.get("sm_mhz") or measured_peaks()[0].get("sm_max_mhz", 1980.0)
     roofline = alu_roofline(float(np.mean(a_v)), 4 * B, atoms_ms / 1e3, "fp64" if form == "fp64" else "fp32",
-                            "atoms_kernel", "cluster, CG, Krylov basis and projection, counted as plain (not pair) arithmetic",
+                            "chains_kernel (atoms_kernel on what it leaves)", "cluster, CG, Krylov basis and projection, counted as plain (not pair) arithmetic",
                             sms, mhz)
     roofline_red = alu_roofline(float(np.mean(a_r)), 4 * B, red_ms / 1e3, "fp64", "reduced_kernel",
                                 "Cholesky, congruence, tridiagonalisation, QL eigenvalues, inverse iteration, "
                                 "back-transform, outputs: 17/3 nu^3 + 47 nu^2 FLOP per column", sms, mhz)
     if form == "mixed":   # DRAM bytes per launch from the profiler capture (null once the kernel has changed)
-        roofline["traffic"] = captured_traffic("atoms_kernel", B)
+        roofline["traffic"] = captured_traffic("chains_kernel", B)
         roofline_red["traffic"] = captured_traffic("reduced_kernel", 4 * B)
     mka.mka_system_destroy(sysh)
     if net is not None:
