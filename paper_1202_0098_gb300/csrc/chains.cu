@@ -44,6 +44,7 @@
 #include <type_traits>
 
 #include "atoms.cuh"
+#include "gram_stage.cuh"
 #include "mka_internal.h"
 
 namespace mka {
@@ -500,10 +501,6 @@ __device__ __noinline__ void gram(const T* W, const T* HW, const T* SW, int m, i
   }
 }
 
-// Floats between the vectors of a chunk of rc rows: an odd number of 16-byte groups, so that eight vectors in a
-// row start in different banks.
-__host__ __device__ constexpr int chunk_stride(int rc) { return 4 * (rc | 1); }
-
 // gram_s: S_r of the FP32 form. Read vector by vector from the slot it was bound by L2 (3.8 MB an atom at nu = 30);
 // here chunks of rows of every vector pass through shared memory once (double buffered, cp.async), and a warp
 // holds two vectors nn against all mm: lane (t, c) has mm = t, t + 8, ... of column c. Sums of eight rows are FP32,
@@ -514,9 +511,7 @@ __device__ __noinline__ void gram_s(const float* W, const float* SW, int m, int 
                                     int64_t col0, double* Gs, int gs_stride, float* stage, int stage_floats) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const int t = lane >> 2, c = lane & 3;
-  const int nvec = n1 + (n1 - n0);             // W 0..n1, then SW n0..n1
-  int rc = 32;                                  // rows of a chunk: two buffers fit
-  while (rc > 4 && 2 * nvec * chunk_stride(rc) > stage_floats) rc -= 4;
+  const int nvec = chunk_vectors(n0, n1), rc = chunk_rows(nvec, stage_floats);
   const int vs = chunk_stride(rc), nchunk = (m + rc - 1) / rc, npair = (n1 - n0 + 1) / 2;
   auto fetch = [&](int k) {
     float* dst = stage + (k & 1) * nvec * vs;
@@ -531,6 +526,9 @@ __device__ __noinline__ void gram_s(const float* W, const float* SW, int m, int 
   for (int j0 = 0; j0 < npair; j0 += nwarp) {
     const int nn = n0 + 2 * (j0 + wid), nb = min(nn + 1, n1 - 1);
     const int cnt = nn < n1 ? nb / 8 + 1 : 0;
+    int at[NA];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) at[i] = lane_vector(t, i, nb) * vs;
     Pair tot[2][NA];
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
@@ -550,7 +548,6 @@ __device__ __noinline__ void gram_s(const float* W, const float* SW, int m, int 
         const float* w = stage + (k & 1) * nvec * vs + c;
         const float* s0 = w + (n1 + nn - n0) * vs;
         const float* s1 = w + (n1 + nb - n0) * vs;
-        w += t * vs;
         const int rows = min(rc, m - k * rc);
         for (int rb = 0; rb < rows; rb += 8) {
           float p0[NA], p1[NA];
@@ -562,7 +559,7 @@ __device__ __noinline__ void gram_s(const float* W, const float* SW, int m, int 
 #pragma unroll
             for (int i = 0; i < NA; ++i)
               if (i < cnt) {
-                const float x = w[8 * i * vs + 4 * r];   // vectors beyond nn + 1 (never beyond the buffer) are unused
+                const float x = w[at[i] + 4 * r];
                 p0[i] = fmaf(x, a, p0[i]);
                 p1[i] = fmaf(x, b, p1[i]);
               }
@@ -597,15 +594,6 @@ struct ChainState {
   double be[4], ga[4], s0[4];    // beta_{n-1}, alpha_n; ||s_j||^2, then beta_p
   int t0, flag, bad, drop, careful;
 };
-
-// Floats of Gs and gv, 16-byte aligned.
-__host__ __device__ constexpr int gs_floats(int p) { return (4 * p * (p + 1) + 8 * p + 3) / 4 * 4; }
-// Shared vectors of m rows hold the seam's Gs, gv and (FP32) two chunks of at least four rows of the p vectors and
-// of all nu.
-__host__ __device__ constexpr bool chains_fit(int m, int p, int nu, bool pairs) {
-  return pairs ? gs_floats(p) + 4 * p * chunk_stride(4) <= 12 * m && 4 * nu * chunk_stride(4) <= 12 * m
-               : gs_floats(p) <= 16 * m;
-}
 
 // The second chain's scalars of column c from beta_p, q.v_k and z.v_k.
 template <typename N>
