@@ -592,7 +592,10 @@ struct ChainState {
   double rr[4], alpha[4], cg_stop[4];
   int it[4], cg_active[4], status[4], fell[4];
   double be[4], ga[4], s0[4];    // beta_{n-1}, alpha_n; ||s_j||^2, then beta_p
-  int t0, flag, bad, drop, careful;
+  // bad: the atom goes to the general kernel, found by the threads that own the scalars between two barriers, so that
+  // it may be read after the second. over: the same, found by the rows' threads as they write a vector; read only
+  // behind the barrier that ends a step.
+  int t0, flag, bad, over, drop, careful;
 };
 
 // The second chain's scalars of column c from beta_p, q.v_k and z.v_k.
@@ -611,7 +614,7 @@ constexpr double kOverlapMax = 1e-3;           // |w_n . e_j| beyond which an at
 constexpr double kOverlapExact = 1e-10;
 
 __device__ __forceinline__ void check_overlap(ChainState& st, double x) {
-  if (!(fabs(x) <= kOverlapMax)) st.bad = 1;
+  if (!(fabs(x) <= kOverlapMax)) st.over = 1;
   if (!(fabs(x) <= kOverlapExact)) st.careful = 1;
 }
 
@@ -695,6 +698,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
         st.t0 = find_local(cl, ncl, (int)atom);
         st.flag = lrow[ncl] <= A.lnnz_cap;
         st.bad = 0;
+        st.over = 0;
         st.drop = 0;
         st.careful = 0;
       }
@@ -1004,7 +1008,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
     // scalars: sc[0..3] beta_{n-1} / eta_k; sc[4..7] alpha_n / h_k, then 1 / beta_n; sc[8..11] s_j.q_n in the
     // first chain; in the second sc[8..11] beta (q.v_k), sc[12..15] beta (z.v_k), sc[16..19] q.v_k, sc[20..23] -z.v_k
     const int q_dim = A.q;
-    for (int n = 0; n < nu && !st.bad; ++n) {
+    for (int n = 0; n < nu && !st.bad && !st.over; ++n) {
       const bool second = n >= A.p && !st.drop;
       const bool last = n == nu - 1;
       const bool with_s = n < A.p && q_dim > 0;
@@ -1304,7 +1308,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
       __syncthreads();
     }
     __syncthreads();
-    if (st.bad) {
+    if (st.bad || st.over) {
       if (tid == 0) A.redo[atomicAdd(A.redo_count, 1)] = (int32_t)widx;
       __syncthreads();
       continue;
