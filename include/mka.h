@@ -251,10 +251,11 @@ void mka_result_destroy(mka_result* res);
 /* Chemical potential (Sec. 2, after Eq. EQ-DM): the mu with
  * 2 sum_j sum_alpha f(eps_alpha^(j); mu) w_alpha^(j) = n_electrons over the
  * result's columns, f(x) = 1 / (1 + exp((x - mu) / kT)). Bracket
- * [min eps - 40 kT, max eps + 40 kT], narrowed by the root finder of
- * mka_sweep_find_mu until no wider than `tol` (eV) or for about 200 steps;
- * returns the midpoint in *mu_out (host). Runs on the device with FP64 sums;
- * synchronises. */
+ * [min eps - 40 kT, max eps + 40 kT], narrowed by bisection and, near the
+ * root, the Illinois secant until no wider than `tol` (eV) or for about 200
+ * steps; returns the midpoint in *mu_out (host). Where several mu give
+ * n_electrons (a gap, full or empty bands) it is the lowest of them, as
+ * bisection alone gives. Runs on the device with FP64 sums; synchronises. */
 mka_status mka_find_mu(mka_result* res, double n_electrons, double kT, double tol, double* mu_out);
 
 /* Density matrix (Eq. EQ-DM) on the selected rows' pattern, the band energy
@@ -370,7 +371,7 @@ mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_p
  * and the batch is enqueued as one CUDA graph (captured the first time this
  * (n_sel, n_electrons, kT, rho_out) combination is seen, replayed afterwards):
  * copy-in, optional ordering by cluster size, the persistent per-atom kernel,
- * up to 64 root-finder steps for mu on the device (as mka_find_mu, tolerance 1e-12 eV),
+ * up to 65 root-finder steps for mu on the device (as mka_find_mu, tolerance 1e-12 eV),
  * rho into `rho_out` (device, [n_blocks][4][4] as in mka_density_energy, may be
  * NULL) and the band energy. Returns without waiting for the GPU; the call waits
  * only for the previous batch to have read the staging buffer. */

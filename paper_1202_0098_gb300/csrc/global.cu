@@ -2,8 +2,8 @@
 // energy, the subspace Green's function, and the global block-sparse product.
 //
 // mu (Sec. 2, after Eq. EQ-DM): the electron count 2 sum_j sum_alpha f w is evaluated by one launch per step of a
-// bracketing root finder (mu_root.cuh: a few bisection steps, then the Illinois secant, 10 to 15 passes where
-// halving alone took 46); the launch's blocks write fixed-order partial sums, and the last block to finish
+// bracketing root finder (mu_root.cuh: a few bisection steps, then the Illinois secant, 10 to 15 passes on metallic
+// levels where halving alone took 46, which a gap still takes); the launch's blocks write fixed-order partial sums, and the last block to finish
 // (ticket counter) adds them in a fixed tree and takes the step, so the result does not depend on timing.
 // f(x) = (1 - tanh((x - mu) / (2 kT))) / 2; for |x - mu| / (2 kT) > 20 the FP64
 // tanh is exactly +-1, so those terms take f = 0 or 1 without calling it.
@@ -120,6 +120,7 @@ __global__ void eps_range_kernel(const double* eps, const double* w, int64_t n, 
       S->fhi = 0.0;
       S->side = 0.0;
       S->rf = 0.0;
+      S->probed = 0.0;
       S->iters = 0;
       *ticket = 0;
     }
@@ -130,7 +131,7 @@ __global__ void eps_range_kernel(const double* eps, const double* w, int64_t n, 
 // Measured at 32,768 columns of nu = 30: 81 us a halving (46 of them) when threads ran over single levels and one
 // thread added the blocks' sums; the whole search now takes 0.4 ms of a batch instead of 5.2.
 __global__ void __launch_bounds__(kRedThreads) mu_pass_kernel(const double* eps, const double* w, int64_t n_cols, int nu,
-                                                              double* partial, unsigned* ticket, RootState* S) {
+                                                              double* partial, unsigned* ticket, RootState* S, int left) {
   __shared__ double red[kRedThreads / 32];
   __shared__ bool last;
   if (!(S->hi - S->lo > S->tol)) return;   // converged: every block leaves before touching the ticket
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(kRedThreads) mu_pass_kernel(const double* eps,
     for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) t += partial[k];
     t = block_sum(t, red);
     if (threadIdx.x == 0) {
-      root_step(S, 2.0 * t);
+      root_step_lowest(S, 2.0 * t, left);
       *ticket = 0;
     }
   }
@@ -670,7 +671,7 @@ mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n_cols, i
   mu_init_kernel<<<1, 1, 0, st>>>(S, ticket, n_electrons, kT, tol);
   eps_range_kernel<<<blocks_of(n_cols * nu), kRedThreads, 0, st>>>(eps, w, n_cols * nu, partial, ticket, S);
   for (int i = 0; i < passes; ++i)
-    mu_pass_kernel<<<blocks_of(n_cols), kRedThreads, 0, st>>>(eps, w, n_cols, nu, partial, ticket, S);
+    mu_pass_kernel<<<blocks_of(n_cols), kRedThreads, 0, st>>>(eps, w, n_cols, nu, partial, ticket, S, passes - 1 - i);
   mu_finish_kernel<<<1, 1, 0, st>>>(S, mu_dev_out);
   count_launches(3 + passes);
   MKA_CUDA_TRY(cudaGetLastError());
@@ -717,12 +718,13 @@ mka_status launch_find_mu(mka_result* res, double n_electrons, double kT, double
   MKA_CUDA_TRY(cudaGetLastError());
   // sixteen passes usually end the search (those after convergence return at once); the bracket comes back and
   // more follow while it is wider than tol
+  constexpr int kBatch = 16, kTotal = 13 * kBatch;
   RootState h{};
-  for (int done = 0; done < 200; done += 16) {
-    for (int i = 0; i < 16; ++i)
+  for (int done = 0; done < kTotal; done += kBatch) {
+    for (int i = 0; i < kBatch; ++i)
       mu_pass_kernel<<<blocks_of(res->n_cols), kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, partial,
-                                                                     ticket, S);
-    count_launches(16);
+                                                                     ticket, S, kTotal - 1 - done - i);
+    count_launches(kBatch);
     MKA_CUDA_TRY(cudaGetLastError());
     MKA_CUDA_TRY(cudaMemcpyAsync(&h, S, sizeof(RootState), cudaMemcpyDeviceToHost, st));
     MKA_CUDA_TRY(cudaStreamSynchronize(st));

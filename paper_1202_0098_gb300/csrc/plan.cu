@@ -30,7 +30,9 @@ namespace mka {
 namespace {
 
 constexpr int kSizeBins = MKA_MAX_CLUSTER_ATOMS + 1;
-constexpr int kMuPasses = 64;   // the root finder needs 10 to 15; 64 halvings alone would close a bracket of 1.8e7 eV to 1e-12
+// The root finder needs 10 to 15 passes on metallic levels, some 50 in a gap; one at the bracket's upper end and 64
+// halvings, which it falls back to, close a bracket of 1.8e7 eV to 1e-12.
+constexpr int kMuPasses = 65;
 
 __global__ void size_hist_kernel(const int32_t* sizes, int64_t n, int32_t* bins) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
