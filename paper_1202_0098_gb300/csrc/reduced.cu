@@ -23,6 +23,7 @@
 #include <stdint.h>
 
 #include "mka_internal.h"
+#include "reduced_rule.cuh"
 
 namespace mka {
 namespace {
@@ -432,7 +433,6 @@ struct Scratch {
   __device__ double& lam(int k) const { return z[(size_t)(4 * nu + k) * 32]; }
 };
 __device__ __forceinline__ Scratch scratch_of(const Lane& M) { return Scratch{&M.Z(0, 0), M.nu}; }
-constexpr int kTeamMinNu = 5;   // the scratch has nu^2 doubles
 
 template <int CPW>
 __device__ __forceinline__ double team_sum(double v) {
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(32) ql_kernel(const RedArgs A) {
 // grow by at most 2.5 a row; a pair below 2^-333 is scaled up again, looked at every 8 rows; a zero counts as a distance
 // of 2^-60, far below the rounding of d_i. QL is one serial chain a column and an FP64 instruction holds a warp's scheduler for 64 cycles: 1.3 ms
 // at nu = 30 and 15 ms at nu = 100, whatever the number of columns; four FP64 operations a row and step make this
-// the shorter way (0.33 ms for 4 columns at nu = 30, 1.2 ms for 148 at nu = 100) up to kFewColumns, and the longer one
+// the shorter way (0.33 ms for 4 columns at nu = 30, 1.2 ms for 148 at nu = 100) for few columns, and the longer one
 // beyond (six times the operations).
 __global__ void __launch_bounds__(32) bisect_kernel(const RedArgs A) {
   extern __shared__ double sm[];
@@ -955,20 +955,9 @@ __global__ void __launch_bounds__(32) team_vectors_kernel(const RedArgs A) {
   }
 }
 
-// Which form (milliseconds measured at nu = 30 / 40; lane: one lane per column):
-//   up to 2,048 columns a whole warp takes a column, the chip is not full (2,048: 2.8 against 9.3);
-//   then teams: 11,996 columns 6.4 against 10.8, 16,384 7.1 against 10.8, 32,768 14.3 against 15.9 (nu = 30);
-//   10,004 columns 15 against 23.9 (nu = 40);
-//   one lane per column once there are enough of them to fill the chip that way, it has no idle lanes (524,288
-//   columns of nu = 30: 158, 0.30 us a column against the teams' 0.44): from about 40,000 columns up to nu = 32, and
-//   16,000 up to nu = 64, where a lane's rate is 0.7 us and a team's 1.5;
-//   nu up to 160 (the packed triangles fit in shared memory): four warps, then a warp per column at any count (148 columns
-//   of nu = 100: 9 against 445); below nu = 5 the scratch between the three kernels does not fit.
-constexpr int64_t kFewColumns = 2048, kManyColumns32 = 40960, kManyColumns64 = 16384;
-
 // TL1 lanes a column in the first kernel, TL2 in the last; nu <= TL NS.
 template <int TL1, int NS1, int TL2, int NS2>
-mka_status team_launch(const RedArgs& A, cudaStream_t st) {
+mka_status team_launch(const RedArgs& A, ReducedForm form, cudaStream_t st) {
   constexpr int C1 = TL1 > 32 ? 1 : 32 / TL1, C2 = 32 / TL2;
   auto k1 = team_tridiag_kernel<TL1, NS1>;
   auto k2 = team_vectors_kernel<TL2, NS2>;
@@ -979,7 +968,7 @@ mka_status team_launch(const RedArgs& A, cudaStream_t st) {
   if (s) return s;
   const size_t smem = sizeof(double) * team_doubles(A.nu);
   k1<<<(unsigned)((A.n_cols + C1 - 1) / C1), TL1 > 32 ? TL1 : 32, smem * C1, st>>>(A);
-  if (A.n_cols <= kFewColumns)
+  if (form == RF_FEW)
     bisect_kernel<<<(unsigned)(A.n_cols * ((A.nu + 31) / 32)), 32, sizeof(double) * 2 * A.nu, st>>>(A);
   else
     ql_kernel<<<(unsigned)((A.n_cols + 31) / 32), 32, sizeof(double) * 2 * A.nu * 32, st>>>(A);
@@ -1004,15 +993,11 @@ mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, 
   A.w = w;
   A.cv = cv;
   A.col0 = col0;
-  if (nu >= kTeamMinNu && nu <= 160) {
-    if (nu > 64) return team_launch<128, 2, 32, 5>(A, st);
-    if (nu > 32) {
-      if (n_cols <= kFewColumns) return team_launch<32, 2, 32, 2>(A, st);
-      if (n_cols <= kManyColumns64) return team_launch<16, 4, 32, 2>(A, st);
-    } else {
-      if (n_cols <= kFewColumns) return team_launch<32, 1, 32, 1>(A, st);
-      if (n_cols <= kManyColumns32) return team_launch<8, 4, 16, 2>(A, st);
-    }
+  const ReducedForm form = reduced_form(nu, n_cols);
+  if (form != RF_LANES) {
+    if (nu > 64) return team_launch<128, 2, 32, 5>(A, form, st);
+    if (nu > 32) return form == RF_FEW ? team_launch<32, 2, 32, 2>(A, form, st) : team_launch<16, 4, 32, 2>(A, form, st);
+    return form == RF_FEW ? team_launch<32, 1, 32, 1>(A, form, st) : team_launch<8, 4, 16, 2>(A, form, st);
   }
   const int threads = 128;
   const unsigned blocks = (unsigned)((n_cols + threads - 1) / threads);
