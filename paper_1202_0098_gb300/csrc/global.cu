@@ -20,6 +20,7 @@
 
 #include "kept.cuh"
 #include "mka_internal.h"
+#include "spmv_rule.cuh"
 #include "widen.cuh"
 #include "mu_root.cuh"
 
@@ -446,48 +447,53 @@ __global__ void __launch_bounds__(kSpmvThreads, (kSpmvBlocks<TX, K>))
   }
 }
 
-// BF16 values with one or two FP32 vectors on large systems: a thread per row, four blocks in flight. A block is 32 bytes
-// there and a load by slots half as wide as the lanes could take, so that the instructions of the kernel above bound it, not
-// memory (262,144 / 5.8 million atoms: one vector 38 / 784 us by slots, 32 / 697 by rows; two 42 / 875 and 42 / 813; four
-// 68 / 1,466 and 73 / 1,550).
-template <int K>
-__global__ void __launch_bounds__(256) spmv_bf16_rows_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                                                             const __nv_bfloat16* __restrict__ val,
-                                                             const float* __restrict__ x, float* __restrict__ y, int64_t n_rows) {
+// A thread per row, its blocks four at a time with their loads in flight: the form for short rows, where most slots
+// of the kernel above would be idle, for many rows of FP64 values, and for BF16 values with one or two FP32 vectors on large
+// systems, where a block is 32 bytes and a load by slots half as wide as the lanes could take (spmv_rule.cuh).
+template <typename TV, typename TX, int K>
+__global__ void __launch_bounds__(256) spmv_rows_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+                                                        const TV* __restrict__ val, const TX* __restrict__ x,
+                                                        TX* __restrict__ y, int64_t n_rows) {
+  using TL = typename std::conditional<std::is_same<TV, double>::value, double, float>::type;
+  auto entry = [](TL v) {
+    if constexpr (sizeof(TX) > sizeof(TL)) return widen(v);
+    else return (TX)v;
+  };
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < 4 * n_rows; g += stride) {
     const int64_t a = g >> 2;
     const int i = (int)(g & 3);
     const int k0 = __ldg(row_ptr + a), k1 = __ldg(row_ptr + a + 1);
-    float acc[K];
+    TX acc[K];
 #pragma unroll
-    for (int c = 0; c < K; ++c) acc[c] = 0.0f;
+    for (int c = 0; c < K; ++c) acc[c] = 0;
     int k = k0;
     for (; k + 4 <= k1; k += 4) {
       int cb[4];
-      float v[4][4];
+      TL v[4][4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) cb[u] = __ldg(col + k + u);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) RowVals<__nv_bfloat16>::load(val, k + u, i, v[u]);
+      for (int u = 0; u < 4; ++u) RowVals<TV>::load(val, k + u, i, v[u]);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        float xv[4][K];
-        load_x<float, K>(x, cb[u], xv);
+        TX xv[4][K];
+        load_x<TX, K>(x, cb[u], xv);
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj)
 #pragma unroll
-          for (int c = 0; c < K; ++c) acc[c] = fmaf(v[u][jj], xv[jj][c], acc[c]);
+          for (int c = 0; c < K; ++c) acc[c] = fma(entry(v[u][jj]), xv[jj][c], acc[c]);
       }
     }
     for (; k < k1; ++k) {
-      float v[4], xv[4][K];
-      RowVals<__nv_bfloat16>::load(val, k, i, v);
-      load_x<float, K>(x, __ldg(col + k), xv);
+      TL v[4];
+      TX xv[4][K];
+      RowVals<TV>::load(val, k, i, v);
+      load_x<TX, K>(x, __ldg(col + k), xv);
 #pragma unroll
       for (int jj = 0; jj < 4; ++jj)
 #pragma unroll
-        for (int c = 0; c < K; ++c) acc[c] = fmaf(v[jj], xv[jj][c], acc[c]);
+        for (int c = 0; c < K; ++c) acc[c] = fma(entry(v[jj]), xv[jj][c], acc[c]);
     }
 #pragma unroll
     for (int c = 0; c < K; ++c) y[g * K + c] = acc[c];
@@ -502,39 +508,43 @@ void spmv_launch(const mka_system* s, const TV* val, const TX* x, TX* y, int sms
       s->d_row_ptr, s->d_col, val, x, y, s->n_atoms);
 }
 
-template <typename TV, typename TX>
-mka_status spmv_dispatch_k(const mka_system* s, const TV* val, const void* x, void* y, int k, cudaStream_t st) {
+template <typename TV, typename TX, int K>
+mka_status spmv_dispatch_k(const mka_system* s, const TV* val, const TX* x, TX* y, cudaStream_t st) {
   int dev = 0, sms = 0;
   MKA_CUDA_TRY(cudaGetDevice(&dev));
   MKA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const TX* xx = reinterpret_cast<const TX*>(x);
-  TX* yy = reinterpret_cast<TX*>(y);
-  if constexpr (std::is_same<TV, __nv_bfloat16>::value && sizeof(TX) == 4)
-    if (k <= 2 && s->n_atoms >= (k == 1 ? 65536 : 131072)) {   // below, both take the same time or the slots less
-      const int64_t blocks = std::min<int64_t>((4 * s->n_atoms + 255) / 256, (int64_t)sms * 8);
-      if (k == 1) spmv_bf16_rows_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
-      else spmv_bf16_rows_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, xx, yy, s->n_atoms);
-      count_launches();
-      MKA_CUDA_TRY(cudaGetLastError());
-      return MKA_OK;
-    }
   // Four slots waste less on rows of 13 blocks and add less (FP64, K = 4, 262,144 atoms: 492 against 539 us); eight spread
   // a small system over more warps (512 atoms, K = 4: 8.8 against 10.9 us; 4,096 atoms, K = 1: 12.9 against 15). They meet at
   // about eight warps an SM.
-  const bool wide = s->n_atoms * k < (int64_t)sms * 64;
-  if (k == 1) wide ? spmv_launch<TV, TX, 1, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 1, 4>(s, val, xx, yy, sms, st);
-  else if (k == 2) wide ? spmv_launch<TV, TX, 2, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 2, 4>(s, val, xx, yy, sms, st);
-  else wide ? spmv_launch<TV, TX, 4, 8>(s, val, xx, yy, sms, st) : spmv_launch<TV, TX, 4, 4>(s, val, xx, yy, sms, st);
+  const bool wide = s->n_atoms * K < (int64_t)sms * 64;
+  if (spmv_by_rows(s->storage == MKA_FP64 ? 0 : s->storage == MKA_MIXED_FP32 ? 1 : 2, sizeof(TX) == 8, K, s->n_atoms, s->nnzb,
+                   wide)) {
+    const int64_t blocks = std::min<int64_t>((4 * s->n_atoms + 255) / 256, (int64_t)sms * 8);
+    spmv_rows_kernel<TV, TX, K><<<(unsigned)blocks, 256, 0, st>>>(s->d_row_ptr, s->d_col, val, x, y, s->n_atoms);
+  } else if (wide) {
+    spmv_launch<TV, TX, K, 8>(s, val, x, y, sms, st);
+  } else {
+    spmv_launch<TV, TX, K, 4>(s, val, x, y, sms, st);
+  }
   count_launches();
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
 }
 
+template <typename TV, typename TX>
+mka_status spmv_dispatch_x(const mka_system* s, const TV* val, const void* x, void* y, int k, cudaStream_t st) {
+  const TX* xx = reinterpret_cast<const TX*>(x);
+  TX* yy = reinterpret_cast<TX*>(y);
+  if (k == 1) return spmv_dispatch_k<TV, TX, 1>(s, val, xx, yy, st);
+  if (k == 2) return spmv_dispatch_k<TV, TX, 2>(s, val, xx, yy, st);
+  return spmv_dispatch_k<TV, TX, 4>(s, val, xx, yy, st);
+}
+
 template <typename TV>
 mka_status spmv_dispatch(const mka_system* s, const void* val, int x_dtype, const void* x, void* y, int k,
                          cudaStream_t st) {
-  if (x_dtype == MKA_FP64) return spmv_dispatch_k<TV, double>(s, (const TV*)val, x, y, k, st);
-  return spmv_dispatch_k<TV, float>(s, (const TV*)val, x, y, k, st);
+  if (x_dtype == MKA_FP64) return spmv_dispatch_x<TV, double>(s, (const TV*)val, x, y, k, st);
+  return spmv_dispatch_x<TV, float>(s, (const TV*)val, x, y, k, st);
 }
 
 // ---- density of states: D(E) = -(1/pi) Im sum_j (G(E + i eta) S)_jj = (eta/pi) sum w / ((E - eps)^2 + eta^2) ----
