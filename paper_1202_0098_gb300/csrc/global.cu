@@ -128,18 +128,29 @@ __global__ void eps_range_kernel(const double* eps, const double* w, int64_t n, 
   }
 }
 
-// One step of the root finder: N(x) = 2 sum f(eps; x) w over the columns (a thread per column), then the bracket.
+// Lanes that share a column's levels: one where the columns fill the chip, up to 32 where they are few and a thread's
+// serial levels are what a pass takes.
+int lanes_per_column(int64_t n_cols) {
+  int l = 1;
+  while (l < 32 && n_cols * l * 2 <= 65536) l *= 2;
+  return l;
+}
+
+// One step of the root finder: N(x) = 2 sum f(eps; x) w over the columns (`share` threads per column), then the bracket.
 // Measured at 32,768 columns of nu = 30: 81 us a halving (46 of them) when threads ran over single levels and one
-// thread added the blocks' sums; the whole search now takes 0.4 ms of a batch instead of 5.2.
+// thread added the blocks' sums; the whole search now takes 0.4 ms of a batch instead of 5.2. Whole columns a thread at 4
+// columns of nu = 100: 681 us a search, 221 with the levels shared.
 __global__ void __launch_bounds__(kRedThreads) mu_pass_kernel(const double* eps, const double* w, int64_t n_cols, int nu,
-                                                              double* partial, unsigned* ticket, RootState* S, int left) {
+                                                              int share, double* partial, unsigned* ticket, RootState* S, int left) {
   __shared__ double red[kRedThreads / 32];
   __shared__ bool last;
   if (!(S->hi - S->lo > S->tol)) return;   // converged: every block leaves before touching the ticket
   const double x = S->x, rk = 0.5 / S->kT;
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cols; i += (int64_t)gridDim.x * blockDim.x)
-    acc += column_count(eps + i * nu, w + i * nu, nu, x, rk);
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_cols * share; t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = t / share;
+    acc += column_count(eps + i * nu, w + i * nu, nu, x, rk, (int)(t % share), share);
+  }
   const double s = block_sum(acc, red);
   if (threadIdx.x == 0) {
     partial[blockIdx.x] = s;
@@ -254,13 +265,15 @@ __global__ void sum_kernel(const double* x, int64_t n, double* out) {
 
 // 2 sum f(eps; mu) w over the columns: per-block partial sums (fixed grid), added by sum_kernel.
 __global__ void __launch_bounds__(kRedThreads) count_partial_kernel(const double* eps, const double* w, int64_t n_cols,
-                                                                    int nu, double mu_host, const double* mu_dev,
-                                                                    double kT, double* partial) {
+                                                                    int nu, int share, double mu_host,
+                                                                    const double* mu_dev, double kT, double* partial) {
   __shared__ double red[kRedThreads / 32];
   const double mu = mu_dev ? *mu_dev : mu_host, rk = 0.5 / kT;
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cols; i += (int64_t)gridDim.x * blockDim.x)
-    acc += column_count(eps + i * nu, w + i * nu, nu, mu, rk);
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_cols * share; t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = t / share;
+    acc += column_count(eps + i * nu, w + i * nu, nu, mu, rk, (int)(t % share), share);
+  }
   const double s = block_sum(acc, red);
   if (threadIdx.x == 0) partial[blockIdx.x] = 2.0 * s;
 }
@@ -680,8 +693,10 @@ mka_status find_mu_enqueue(const double* eps, const double* w, int64_t n_cols, i
   unsigned* ticket = reinterpret_cast<unsigned*>(partial + 2 * kMaxRedBlocks);
   mu_init_kernel<<<1, 1, 0, st>>>(S, ticket, n_electrons, kT, tol);
   eps_range_kernel<<<blocks_of(n_cols * nu), kRedThreads, 0, st>>>(eps, w, n_cols * nu, partial, ticket, S);
+  const int share = lanes_per_column(n_cols);
   for (int i = 0; i < passes; ++i)
-    mu_pass_kernel<<<blocks_of(n_cols), kRedThreads, 0, st>>>(eps, w, n_cols, nu, partial, ticket, S, passes - 1 - i);
+    mu_pass_kernel<<<blocks_of(n_cols * share), kRedThreads, 0, st>>>(eps, w, n_cols, nu, share, partial, ticket, S,
+                                                                      passes - 1 - i);
   mu_finish_kernel<<<1, 1, 0, st>>>(S, mu_dev_out);
   count_launches(3 + passes);
   MKA_CUDA_TRY(cudaGetLastError());
@@ -695,7 +710,8 @@ mka_status density_enqueue(const mka_system* sys, const int64_t* sel, const int6
                                                   sys->storage, nu, 0.0, mu_dev, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, n_sel, tmp + n_sel);
   const int rb = red_blocks();
-  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(eps, w, 4 * n_sel, nu, 0.0, mu_dev, kT, tmp + n_sel + 2);
+  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(eps, w, 4 * n_sel, nu, lanes_per_column(4 * n_sel), 0.0, mu_dev, kT,
+                                                    tmp + n_sel + 2);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp + n_sel + 2, rb, tmp + n_sel + 1);
   count_launches(4);
   MKA_CUDA_TRY(cudaGetLastError());
@@ -729,11 +745,12 @@ mka_status launch_find_mu(mka_result* res, double n_electrons, double kT, double
   // sixteen passes usually end the search (those after convergence return at once); the bracket comes back and
   // more follow while it is wider than tol
   constexpr int kBatch = 16, kTotal = 13 * kBatch;
+  const int share = lanes_per_column(res->n_cols);
   RootState h{};
   for (int done = 0; done < kTotal; done += kBatch) {
     for (int i = 0; i < kBatch; ++i)
-      mu_pass_kernel<<<blocks_of(res->n_cols), kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, partial,
-                                                                     ticket, S, kTotal - 1 - done - i);
+      mu_pass_kernel<<<blocks_of(res->n_cols * share), kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, share,
+                                                                             partial, ticket, S, kTotal - 1 - done - i);
     count_launches(kBatch);
     MKA_CUDA_TRY(cudaGetLastError());
     MKA_CUDA_TRY(cudaMemcpyAsync(&h, S, sizeof(RootState), cudaMemcpyDeviceToHost, st));
@@ -755,8 +772,8 @@ mka_status launch_density(mka_system* sys, mka_result* res, double mu, double kT
                                                        res->d_sel, sys->d_row_ptr, sys->d_valH, sys->storage,
                                                        res->nu, mu, nullptr, kT, rho_out, tmp);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp, res->n_sel, tmp + res->n_sel);
-  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, mu, nullptr, kT,
-                                                   tmp + res->n_sel + 2);
+  count_partial_kernel<<<rb, kRedThreads, 0, st>>>(res->d_eps, res->d_w, res->n_cols, res->nu, lanes_per_column(res->n_cols), mu,
+                                                   nullptr, kT, tmp + res->n_sel + 2);
   sum_kernel<<<1, kRedThreads, 0, st>>>(tmp + res->n_sel + 2, rb, tmp + res->n_sel + 1);
   count_launches(4);
   cudaError_t e = cudaGetLastError();

@@ -93,14 +93,14 @@ __device__ inline void root_step_lowest(RootState* S, double t, int left) {
   S->rf = rf;
 }
 
-// f w summed over a column's nu levels (ascending; entries with w = 0 add nothing). A thread takes a whole column: at
-// a given level index the lanes of a warp hold levels of much the same energy, so that they agree on whether f
-// is 1, 0 or needs the tanh, which only a quarter of the levels do. rk = 1 / (2 kT).
+// f w summed over a column's levels part, part + step, ... (ascending; entries with w = 0 add nothing). With step = 1
+// a thread takes a whole column: at a given level index the lanes of a warp hold levels of much the same energy, so that
+// they agree on whether f is 1, 0 or needs the tanh, which only a quarter of the levels do. rk = 1 / (2 kT).
 __device__ __forceinline__ double column_count(const double* __restrict__ eps, const double* __restrict__ w, int nu,
-                                               double mu, double rk) {
+                                               double mu, double rk, int part = 0, int step = 1) {
   double c = 0.0;
 #pragma unroll 4
-  for (int a = 0; a < nu; ++a) {
+  for (int a = part; a < nu; a += step) {
     const double wi = w[a], y = (eps[a] - mu) * rk;
     if (wi != 0.0 && !(y > 20.0)) c += (y < -20.0 ? 1.0 : 0.5 * (1.0 - tanh(y))) * wi;
   }
