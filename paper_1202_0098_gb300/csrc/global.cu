@@ -658,7 +658,8 @@ mka_status launch_dos(const double* eps, const double* w, int64_t n, const doubl
   // 8 groups of 32 energies a CTA; with fewer the warps share a group. About four CTAs per SM, 64 to 32,768 levels each.
   const int groups = (n_e + 31) / 32, share = groups >= 8 ? 1 : groups >= 4 ? 2 : groups >= 2 ? 4 : 8;
   const int gy = (groups + kDosWarps / share - 1) / (kDosWarps / share);
-  int64_t chunk = (n * gy + red_blocks() - 1) / red_blocks();
+  const int64_t fill = std::max(1, red_blocks() / gy);   // chunks; one more than fill the SMs evenly costs a fifth
+  int64_t chunk = (n + fill - 1) / fill;
   chunk = std::min<int64_t>(32768, std::max<int64_t>(64, (chunk + 63) / 64 * 64));
   const int64_t n_chunks = std::max<int64_t>(1, (n + chunk - 1) / chunk);
   double* buf = nullptr;
