@@ -443,6 +443,8 @@ mka_status mka_autotune_batch(mka_system* sys, const mka_solve_params* prm, cons
  * Memory: 16 (kp + 1) x 8 bytes per pattern block of the range, plus
  * 16 nu bytes and 2 bytes per column.
  *
+ * An atom's levels do not depend on the batch or the plan size it is swept with:
+ * the kernels are picked by the system's size.
  * Deterministic sums: the electron count, the band energy and the
  * level-energy are summed per chunk of `chunk_atoms` consecutive atoms (chunk g
  * = atoms [g chunk_atoms, (g+1) chunk_atoms) of the whole system) in a fixed

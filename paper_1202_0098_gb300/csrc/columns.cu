@@ -55,6 +55,7 @@
 
 #include "atoms.cuh"
 #include "mka_internal.h"
+#include "reduced_rule.cuh"
 
 namespace mka {
 namespace {
@@ -1151,7 +1152,8 @@ mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl,
 }
 
 mka_status reduced_for(const mka_system* sys, const AtomsLaunchArgs& a, cudaStream_t st) {
-  return reduced_launch(a.red, 4 * a.n_sel, a.p + a.q, a.status, a.nu_eff, a.eps, a.w, a.keep ? a.cv : nullptr,
+  const int nu = a.p + a.q;
+  return reduced_launch(a.red, 4 * a.n_sel, a.pick_atoms ? system_columns(nu, a.pick_atoms) : 4 * a.n_sel, nu, a.status, a.nu_eff, a.eps, a.w, a.keep ? a.cv : nullptr,
                         a.col0, st);
 }
 
@@ -1159,7 +1161,7 @@ mka_status atoms_launch(const mka_system* sys, int arith, const AtomsConfig& cf,
                         cudaStream_t st) {
   const bool mixed = arith != MKA_FP64;
   // few atoms: a CTA per column, from x0 = 0 and without keeping s_j
-  if (a.n_sel <= cf.single_max && !a.cg_only && !a.mode_b && !a.x0 && !a.prev_s && !a.keep_s && !a.fallback && a.grid <= 0)
+  if (std::max(a.pick_atoms, a.n_sel) <= cf.single_max && !a.cg_only && !a.mode_b && !a.x0 && !a.prev_s && !a.keep_s && !a.fallback && a.grid <= 0)
     return single_launch(sys, cf, a, st);
   if (cf.chains) {
     const mka_status s = chains_launch(sys, arith, cf, a, st);

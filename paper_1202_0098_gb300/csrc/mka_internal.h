@@ -116,6 +116,9 @@ struct AtomsLaunchArgs {
   const int64_t* sel = nullptr;    // device selected atoms
   const int32_t* order = nullptr;  // device work order (selection indices) or NULL
   int64_t n_sel = 0;
+  // Atoms by whose number the kernels are picked (0: n_sel). A sweep's batches pick by the whole system's: the forms round
+  // differently, and an atom's levels may not depend on the batch, nor on the process, that it is in.
+  int64_t pick_atoms = 0;
   int p = 0, q = 0;
   double cg_tol = 0;
   int cg_maxit = 0;
@@ -168,7 +171,8 @@ inline size_t red_buffer_bytes(int64_t n_cols, int nu) {
 // The batched reduced problems (reduced.cu): one lane per column over the buffer filled by
 // the per-atom kernel; writes eps, w (ranked), the final status and nu_eff, and (cv != NULL)
 // the kept C and V_j of column col0 + c.
-mka_status reduced_launch(double* red, int64_t n_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
+// pick_cols: columns by whose number the form is picked (reduced_rule.cuh).
+mka_status reduced_launch(double* red, int64_t n_cols, int64_t pick_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
                           double* w, double* cv, int64_t col0, cudaStream_t st);
 
 // Learned warm start (mlp.cu).

@@ -206,6 +206,7 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   a.cv = r->d_cv;
   a.col0 = 0;
   a.mode_b = P->prm.subspace == MKA_SUBSPACE_B;
+  if (m.kind != PLAN_BATCH) a.pick_atoms = P->sys->n_atoms;
   MKA_CUDA_TRY(cudaEventRecordWithFlags(P->k0, st, cudaEventRecordExternal));
   mka_status s = atoms_launch(P->sys, P->prm.arith, P->cf, a, st);
   if (s) return s;

@@ -980,7 +980,7 @@ mka_status team_launch(const RedArgs& A, ReducedForm form, cudaStream_t st) {
 
 }  // namespace
 
-mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
+mka_status reduced_launch(double* blk, int64_t n_cols, int64_t pick_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
                           double* w, double* cv, int64_t col0, cudaStream_t st) {
   if (n_cols <= 0) return MKA_OK;
   RedArgs A{};
@@ -993,7 +993,7 @@ mka_status reduced_launch(double* blk, int64_t n_cols, int nu, int32_t* status, 
   A.w = w;
   A.cv = cv;
   A.col0 = col0;
-  const ReducedForm form = reduced_form(nu, n_cols);
+  const ReducedForm form = reduced_form(nu, pick_cols);
   if (form != RF_LANES) {
     if (nu > 64) return team_launch<128, 2, 32, 5>(A, form, st);
     if (nu > 32) return form == RF_FEW ? team_launch<32, 2, 32, 2>(A, form, st) : team_launch<16, 4, 32, 2>(A, form, st);

@@ -32,4 +32,11 @@ constexpr ReducedForm reduced_form(int nu, int64_t n_cols) {
   return n_cols <= few ? RF_FEW : n_cols <= teams ? RF_TEAMS : RF_LANES;
 }
 
+// The columns a sweep over a system of n atoms picks its form by, whatever its batches are: all of them, so that no batch
+// is slower than with a lane per column, or, from nu = 24 to 32, half: up to twice the limit the teams cost 10 % of these
+// kernels and save up to half in batches below it (55,296 columns of nu = 30 in batches of 16,384: 27 ms against 38).
+constexpr int64_t system_columns(int nu, int64_t n) {
+  return 4 * n > 2048 && nu >= 24 && nu <= 32 ? (2 * n > 2048 ? 2 * n : 2049) : 4 * n;
+}
+
 }  // namespace mka
