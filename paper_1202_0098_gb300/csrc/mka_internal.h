@@ -249,6 +249,13 @@ constexpr int kDensityTmpExtra = kMaxRedBlocks;
 size_t storage_bytes(int storage);
 
 // ---- whole-system sweeps (sweep.cu) ----
+// A number no other sweep or network of this process has had: what a plan's graphs know them by, since a new one may come
+// to lie at a destroyed one's address while the graphs hold the old one's device pointers.
+inline uint64_t next_serial() {
+  static std::atomic<uint64_t> n{0};
+  return ++n;
+}
+uint64_t sweep_serial(const mka_sweep* sw);
 // What a plan does with a batch after its column kernels.
 enum PlanModeKind { PLAN_BATCH = 0, PLAN_SWEEP = 1, PLAN_AT_MU = 2 };
 struct PlanMode {

@@ -61,14 +61,14 @@ __global__ void size_scatter_kernel(const int32_t* sizes, int64_t n, int32_t* bi
 struct GraphEntry {
   int64_t n = 0;
   int kind = PLAN_BATCH;
-  const mka_sweep* sw = nullptr;
+  uint64_t sw = 0;           // serial of the sweep (0: none)
   double n_electrons = 0, kT = 0, mu = 0;
   double* rho = nullptr;
   cudaGraphExec_t exec = nullptr;
   int64_t kernels = 0;
   bool forces = false;
   bool same(int64_t n_, const PlanMode& m) const {
-    return n == n_ && kind == m.kind && sw == m.sw && n_electrons == m.n_electrons && kT == m.kT && mu == m.mu &&
+    return n == n_ && kind == m.kind && sw == (m.sw ? sweep_serial(m.sw) : 0) && n_electrons == m.n_electrons && kT == m.kT && mu == m.mu &&
            rho == m.rho && forces == m.forces;
   }
 };
@@ -376,7 +376,7 @@ mka_status mka::plan_run_mode(mka_plan* P, const int64_t* atoms, int64_t n_sel, 
     GraphEntry ge;
     ge.n = n_sel;
     ge.kind = m.kind;
-    ge.sw = m.sw;
+    ge.sw = m.sw ? sweep_serial(m.sw) : 0;
     ge.n_electrons = m.n_electrons;
     ge.kT = m.kT;
     ge.mu = m.mu;

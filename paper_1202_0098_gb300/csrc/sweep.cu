@@ -454,6 +454,7 @@ size_t pack_smem_bytes(int nu, int kp) { return sizeof(double) * 4 * (size_t)nu 
 }  // namespace mka
 
 struct mka_sweep {
+  const uint64_t serial = mka::next_serial();
   mka_system* sys = nullptr;
   cudaStream_t stream = nullptr;
   int nu = 0, kp = 0;
@@ -947,6 +948,7 @@ mka_status mka_sweep_device_levels(const mka_sweep* sw, const double** eps, cons
 
 namespace mka {
 // Orders a plan's work on `plan_stream` after the sweep's earlier work, and the sweep's later work after it.
+uint64_t sweep_serial(const mka_sweep* sw) { return sw->serial; }
 mka_status sweep_join_before(mka_sweep* sw, cudaStream_t plan_stream) { return join(sw->stream, plan_stream, sw->ev); }
 mka_status sweep_join_after(mka_sweep* sw, cudaStream_t plan_stream) { return join(plan_stream, sw->stream, sw->ev); }
 }  // namespace mka
