@@ -256,6 +256,7 @@ inline uint64_t next_serial() {
   return ++n;
 }
 uint64_t sweep_serial(const mka_sweep* sw);
+uint64_t mlp_serial(const mka_mlp* net);
 // What a plan does with a batch after its column kernels.
 enum PlanModeKind { PLAN_BATCH = 0, PLAN_SWEEP = 1, PLAN_AT_MU = 2 };
 struct PlanMode {

@@ -460,6 +460,7 @@ unsigned blocks_for(int64_t n, int per) { return (unsigned)std::max<int64_t>(1, 
 }  // namespace mka
 
 struct mka_mlp {
+  const uint64_t serial = mka::next_serial();
   float* theta = nullptr;          // FP32 master
   __nv_bfloat16* thetab = nullptr; // BF16 copy used by every product
   float* m = nullptr;
@@ -490,6 +491,8 @@ mka_status rows_enqueue(const RowArgs& A, cudaStream_t st) {
 }
 
 }  // namespace
+
+uint64_t mlp_serial(const mka_mlp* net) { return net->serial; }
 
 mka_status mlp_forward_enqueue(const mka_mlp* net, const float* X, int64_t B, float* Y, cudaStream_t st) {
   RowArgs A{};

@@ -62,13 +62,14 @@ struct GraphEntry {
   int64_t n = 0;
   int kind = PLAN_BATCH;
   uint64_t sw = 0;           // serial of the sweep (0: none)
+  uint64_t net = 0;          // serial of the learned start's network (0: none)
   double n_electrons = 0, kT = 0, mu = 0;
   double* rho = nullptr;
   cudaGraphExec_t exec = nullptr;
   int64_t kernels = 0;
   bool forces = false;
-  bool same(int64_t n_, const PlanMode& m) const {
-    return n == n_ && kind == m.kind && sw == (m.sw ? sweep_serial(m.sw) : 0) && n_electrons == m.n_electrons && kT == m.kT && mu == m.mu &&
+  bool same(int64_t n_, const PlanMode& m, uint64_t net_) const {
+    return n == n_ && net == net_ && kind == m.kind && sw == (m.sw ? sweep_serial(m.sw) : 0) && n_electrons == m.n_electrons && kT == m.kT && mu == m.mu &&
            rho == m.rho && forces == m.forces;
   }
 };
@@ -343,6 +344,9 @@ mka_status mka::plan_run_mode(mka_plan* P, const int64_t* atoms, int64_t n_sel, 
     mka_status sc = sweep_check_atoms(m.sw, sys, P->prm.p + P->prm.q, atoms, n_sel);
     if (sc) return sc;
   }
+  if (P->prm.use_warm_start && !sys->warm)
+    return fail(MKA_ERR_INVALID_ARG, "use_warm_start needs a network attached with mka_system_set_warm_start");
+  const uint64_t net = P->prm.use_warm_start ? mlp_serial(sys->warm) : 0;
   // the previous batch's copies must have read the staging buffer before it is refilled
   MKA_CUDA_TRY(cudaEventSynchronize(P->staged));
   int64_t* off = P->h_stage + P->max_atoms;
@@ -359,7 +363,7 @@ mka_status mka::plan_run_mode(mka_plan* P, const int64_t* atoms, int64_t n_sel, 
   r->h_blk_off.assign(off, off + n_sel + 1);
   GraphEntry* g = nullptr;
   for (auto& e : P->graphs)
-    if (e.same(n_sel, m)) g = &e;
+    if (e.same(n_sel, m, net)) g = &e;
   if (!g) {
     cudaGraph_t graph = nullptr;
     const int64_t k0 = mka_kernel_launches();
@@ -377,6 +381,7 @@ mka_status mka::plan_run_mode(mka_plan* P, const int64_t* atoms, int64_t n_sel, 
     ge.n = n_sel;
     ge.kind = m.kind;
     ge.sw = m.sw ? sweep_serial(m.sw) : 0;
+    ge.net = net;
     ge.n_electrons = m.n_electrons;
     ge.kT = m.kT;
     ge.mu = m.mu;

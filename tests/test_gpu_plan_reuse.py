@@ -32,3 +32,32 @@ def test_sweeps_one_after_the_other(system):
         want = total if want is None else want
         assert abs(total - want) <= 1e-10 * abs(want)
     mka.mka_plan_destroy(plan)
+
+
+def test_networks_one_after_the_other(system):
+    """The learned start's network replaced between runs: every run starts from the one attached then, as a direct solve
+    does; with none attached a plan refuses, as a direct solve does."""
+    mka, s, n = system
+    atoms = np.arange(40, dtype=np.int64)
+    prm = mka.solve_params(4, 4, arith="mixed", cg_tol=1e-7, use_warm_start=True)
+    plan, seen = None, []
+    for i in range(6):
+        net = mka.mka_mlp_create(i)
+        mka.mka_mlp_set_params(net, mka.mka_mlp_get_params(net) * np.float32(0.02 + 0.1 * (i % 3)))
+        mka.mka_system_set_warm_start(s, net)
+        plan = plan or mka.mka_plan_create(s, len(atoms), prm)
+        res = mka.mka_solve_columns(s, atoms, prm)
+        want = mka.mka_result_copy_levels(res)["cg_iters"], mka.mka_result_copy_warm_start(res)
+        mka.mka_result_destroy(res)
+        mka.mka_plan_run(plan, atoms, 4.0 * len(atoms), 0.1)
+        pres = mka.mka_plan_result(plan)
+        np.testing.assert_array_equal(mka.mka_result_copy_levels(pres)["cg_iters"], want[0])
+        np.testing.assert_array_equal(mka.mka_result_copy_warm_start(pres), want[1])
+        seen.append((want[0].sum(), want[1].sum()))
+        mka.mka_system_set_warm_start(s, None)
+        with pytest.raises(mka.MkaError) as e:
+            mka.mka_plan_run(plan, atoms, 4.0 * len(atoms), 0.1)
+        assert e.value.status == mka.MKA_ERR_INVALID_ARG
+        mka.mka_mlp_destroy(net)
+    mka.mka_plan_destroy(plan)
+    assert len(set(seen)) > 1
