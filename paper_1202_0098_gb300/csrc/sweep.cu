@@ -12,10 +12,11 @@
 // column. Atoms whose columns have more than kp levels in the window, and all atoms when mu is
 // outside that range, are solved again at mu.
 //
-// Sums (electron count, band energy) run per chunk of consecutive atoms of the whole system, in a
-// fixed order inside the chunk (blocks of 64 atoms, a thread per column and a fixed tree; then the
-// blocks, a warp per chunk), and the chunk sums are added in chunk order. A process that sweeps a range starting on a chunk boundary therefore reproduces a
-// whole-system process's chunk sums exactly, and the root finder (mu_root.cuh) gives the same mu.
+// Sums (electron count, band energy) run per chunk of consecutive atoms of the whole system, in a fixed order inside the
+// chunk (blocks of 64 atoms, a thread or, in short chunks, several per column and a fixed tree; then the blocks, a
+// warp per chunk), and the chunk sums are added in chunk order. A process that sweeps a range starting on a chunk
+// boundary therefore reproduces a whole-system process's chunk sums exactly, and the root finder (mu_root.cuh) gives
+// the same mu.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -232,6 +233,7 @@ struct ChunkArgs {
   int nu;
   int64_t a0, a1, chunk_atoms, chunk0;
   int n_sub;                 // blocks per chunk
+  int share;                 // threads per column
   double mu;                 // used when S == NULL
   const RootState* S;        // root finder: mu = the state's next point; nothing once converged
   double kT;
@@ -240,7 +242,9 @@ struct ChunkArgs {
   int levels, rho;           // also the level energies / the atoms' 2 sum rho H
 };
 
-// One CTA per block of 64 consecutive atoms of a chunk, a thread per column. One CTA per whole chunk left most
+// One CTA per block of 64 consecutive atoms of a chunk, a thread per column; up to 32 threads share a column where a
+// chunk has fewer atoms, as far as its levels go round (all sums of 1,024 chunks of one atom, nu = 30: 97 us with 4 of 256
+// threads at work, 66 now). One CTA per whole chunk left most
 // of the chip idle (13,824 atoms in chunks of 4,096: four CTAs, 340 us a pass, 69 ms of a 226 ms system; now 2.5 ms), and its threads ran over single
 // levels, a warp's lanes split between f = 1, f = 0 and the tanh.
 __global__ void __launch_bounds__(kChunkThreads) sweep_chunk_kernel(const ChunkArgs A) {
@@ -255,19 +259,25 @@ __global__ void __launch_bounds__(kChunkThreads) sweep_chunk_kernel(const ChunkA
   const int64_t gi = blockIdx.x / A.n_sub, sub = blockIdx.x % A.n_sub;
   const int64_t g0 = (A.chunk0 + gi) * A.chunk_atoms, b0 = g0 + sub * kSubAtoms;
   const int64_t lo = max(A.a0, b0), hi = min(A.a1, min(g0 + A.chunk_atoms, b0 + kSubAtoms));
-  const int64_t atom = b0 + (threadIdx.x >> 2);
+  const int part = (int)threadIdx.x % A.share, lcol = (int)threadIdx.x / A.share;
+  const int64_t atom = b0 + (lcol >> 2);
   double c = 0.0, el = 0.0, er = 0.0;
   if (atom >= lo && atom < hi) {
-    const int64_t col = 4 * (atom - A.a0) + (threadIdx.x & 3);
+    const int64_t col = 4 * (atom - A.a0) + (lcol & 3);
     const double* eps = A.eps + col * A.nu;
     const double* w = A.w + col * A.nu;
-    c = column_count(eps, w, A.nu, mu, rk);
     if (A.levels)
-      for (int a = 0; a < A.nu; ++a) {
-        const double wi = w[a];
-        if (wi != 0.0) el += fermi_f(eps[a], mu, rk) * eps[a] * wi;
+      for (int a = part; a < A.nu; a += A.share) {   // column_count's sum with the level energies beside it
+        const double wi = w[a], x = eps[a];
+        if (wi != 0.0) {
+          const double f = fermi_f(x, mu, rk);
+          c += f * wi;
+          el += f * x * wi;
+        }
       }
-    if (A.rho && (threadIdx.x & 3) == 0) er = A.eatom[atom - A.a0];
+    else
+      c = column_count(eps, w, A.nu, mu, rk, part, A.share);
+    if (A.rho && (lcol & 3) == 0 && part == 0) er = A.eatom[atom - A.a0];
   }
   const double cs = cta_sum(c, red);
   const double es = A.levels ? cta_sum(el, red) : 0.0;
@@ -572,17 +582,20 @@ mka_status chunk_launch(mka_sweep* sw, double mu, double kT, const RootState* S,
   A.chunk_atoms = sw->chunk_atoms;
   A.chunk0 = sw->chunk0;
   A.n_sub = sw->n_sub;
+  A.share = 1;                                  // by the chunk's length and nu alone: the same sums in every process
+  while (A.share < 32 && 2 * A.share <= sw->nu && sw->chunk_atoms <= kSubAtoms / (2 * A.share)) A.share *= 2;
   A.mu = mu;
   A.S = S;
   A.kT = kT;
-  A.part = sw->d_part_sums;
+  A.part = sw->n_sub == 1 ? sw->d_chunk : sw->d_part_sums;   // one block is the chunk
   A.n_chunks = sw->n_chunks;
   A.levels = levels;
   A.rho = rho;
   sweep_chunk_kernel<<<(unsigned)(sw->n_chunks * sw->n_sub), kChunkThreads, 0, sw->stream>>>(A);
-  sweep_fold_kernel<<<(unsigned)((sw->n_chunks + 7) / 8), 256, 0, sw->stream>>>(
-      sw->d_part_sums, sw->n_chunks, sw->n_sub, 1 | (levels ? 2 : 0) | (rho ? 4 : 0), sw->d_chunk, S);
-  count_launches(2);
+  if (sw->n_sub > 1)
+    sweep_fold_kernel<<<(unsigned)((sw->n_chunks + 7) / 8), 256, 0, sw->stream>>>(
+        sw->d_part_sums, sw->n_chunks, sw->n_sub, 1 | (levels ? 2 : 0) | (rho ? 4 : 0), sw->d_chunk, S);
+  count_launches(sw->n_sub > 1 ? 2 : 1);
   MKA_CUDA_TRY(cudaGetLastError());
   return MKA_OK;
 }

@@ -25,6 +25,8 @@ def test_chunk_sums(chunk):
             sw = mka.mka_sweep_create(s, a0, n, nu, 0.0, 4.0, 8, chunk)
             mka.mka_plan_run_sweep(plan, sw, np.arange(a0, n, dtype=np.int64))
             sums.append(mka.mka_sweep_chunk_sums(sw, mu, kT))
+            alone = mka.mka_sweep_chunk_sums(sw, mu, kT, levels=False)["count"]
+            np.testing.assert_array_equal(alone, sums[-1]["count"])
             if a0 == 0:
                 res = mka.mka_plan_result(plan)
                 lv = mka.mka_result_copy_levels(res)
