@@ -403,8 +403,9 @@ void mka_plan_destroy(mka_plan* plan);
  * 512, resident CTAs per SM max/1/2, ordering by cluster size off/on) that fits
  * runs the sample batch (host atoms) three times through a plan, the fastest of
  * the last two timings wins. With `cache_path` (a JSON file, NULL = none) the
- * choice is looked up first under a key of GPU name, storage, arithmetic, p+q,
- * the sample's largest cluster (rounded down to 16) and the sample size, and
+ * choice is looked up first under a key of GPU name, the library's sources (a
+ * choice measured with other kernels is not taken over), storage, arithmetic,
+ * p+q, the sample's largest cluster (rounded down to 16) and the sample size, and
  * stored there after a search. */
 mka_status mka_autotune(mka_system* sys, const mka_solve_params* prm, const int64_t* sample, int64_t n_sample,
                         double n_electrons, double kT, const char* cache_path, void* stream, mka_tuning* out);
@@ -412,7 +413,7 @@ mka_status mka_autotune(mka_system* sys, const mka_solve_params* prm, const int6
 /* Choose the batch size of plans for `prm` and launch shape `tune` (NULL = defaults): each candidate
  * (host array, atoms per batch) that fits runs a batch of consecutive atoms from first_atom through a
  * plan twice; the highest columns/s of the second run wins, into *out_batch. With `cache_path` the
- * choice is looked up first and stored after a search (key: GPU, storage, arithmetic, p + q, subspace,
+ * choice is looked up first and stored after a search (key: GPU, library sources, storage, arithmetic, p + q, subspace,
  * system size, launch shape, candidates). MKA_ERR_OOM when no candidate fits. */
 mka_status mka_autotune_batch(mka_system* sys, const mka_solve_params* prm, const mka_tuning* tune,
                               const int64_t* candidates, int n_candidates, int64_t first_atom,

@@ -8,6 +8,7 @@ paper_1202_0098_gb300/_build/libmka.so (git-ignored).
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import shutil
 import subprocess
@@ -28,6 +29,16 @@ def nvcc() -> str:
     if not os.path.exists(path):
         raise RuntimeError("nvcc not found: the CUDA toolkit is required to build libmka")
     return path
+
+
+def source_mark() -> str:
+    """A short hash of the library's sources: what tuning results are cached under, so that a choice measured with other
+    kernels is not taken over."""
+    h = hashlib.sha256()
+    for f in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, f), "rb") as fh:
+            h.update(f.encode() + b"\0" + fh.read())
+    return h.hexdigest()[:12]
 
 
 def _compile(src: str, extra: list[str]) -> str:
@@ -53,7 +64,7 @@ def build(force: bool = False, verbose: bool = False, extra: list[str] | None = 
     objs = [os.path.join(BUILD, os.path.splitext(s)[0] + ".o") for s in SOURCES]
     if not force and not _stale(objs):
         return LIB
-    extra = list(extra or [])
+    extra = [*(extra or []), f'-DMKA_SOURCE_MARK="{source_mark()}"']
     with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
         objs = list(ex.map(lambda s: _compile(s, extra), SOURCES))
     tmp = LIB + ".tmp"

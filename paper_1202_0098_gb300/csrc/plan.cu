@@ -12,7 +12,7 @@
 //
 // The autotuner times candidate launch shapes (CTA size, resident CTAs per SM,
 // size ordering) on a sample batch and keeps the fastest, optionally cached in a
-// small JSON file keyed by GPU, storage, arithmetic, subspace size and cluster size.
+// small JSON file keyed by GPU, the library's sources, storage, arithmetic, subspace size and cluster size.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -25,6 +25,10 @@
 #include <vector>
 
 #include "mka_internal.h"
+
+#ifndef MKA_SOURCE_MARK           // a hash of the sources, given by the build
+#define MKA_SOURCE_MARK "unknown"
+#endif
 
 namespace mka {
 namespace {
@@ -454,7 +458,7 @@ mka_status mka_autotune(mka_system* sys, const mka_solve_params* prm, const int6
   if (s) return s;
   const int max_cl = *std::max_element(sz.begin(), sz.end());
   std::ostringstream key;
-  key << prop.name << "|storage=" << sys->storage << "|arith=" << prm->arith << "|nu=" << prm->p + prm->q
+  key << prop.name << "|kernels=" << MKA_SOURCE_MARK << "|storage=" << sys->storage << "|arith=" << prm->arith << "|nu=" << prm->p + prm->q
       << "|subspace=" << prm->subspace
       << "|maxcl=" << (max_cl / 16) * 16 << "|nsample=" << n_sample;
   const std::string k = key.str();
@@ -541,7 +545,7 @@ mka_status mka_autotune_batch(mka_system* sys, const mka_solve_params* prm, cons
   MKA_CUDA_TRY(cudaGetDevice(&dev));
   MKA_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
   std::ostringstream key;
-  key << prop.name << "|storage=" << sys->storage << "|arith=" << prm->arith << "|nu=" << prm->p + prm->q
+  key << prop.name << "|kernels=" << MKA_SOURCE_MARK << "|storage=" << sys->storage << "|arith=" << prm->arith << "|nu=" << prm->p + prm->q
       << "|subspace=" << prm->subspace << "|atoms=" << sys->n_atoms << "|threads=" << t.threads
       << "|ctas=" << t.ctas_per_sm << "|order=" << t.order_by_size << "|batch_of";
   for (int i = 0; i < n_candidates; ++i) key << ":" << candidates[i];
