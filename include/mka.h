@@ -363,7 +363,8 @@ typedef struct mka_plan mka_plan; /* every buffer of one batch of the work flow,
  * kept data as for keep_vectors, mu over the batch's columns, rho and the band
  * energy) with every buffer allocated here, once. `tune` may be NULL (defaults,
  * or pass the result of mka_autotune). The plan computes the largest cluster of
- * the whole system once, to size its work slots. Work runs on `stream`. */
+ * the whole system once, to size its work slots, and solves up to 64 atoms spread
+ * over the system to choose between its per-atom kernels. Work runs on `stream`. */
 mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_params* prm,
                            const mka_tuning* tune, void* stream, mka_plan** out);
 

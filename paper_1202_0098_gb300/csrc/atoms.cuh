@@ -81,6 +81,7 @@ struct Args {
   int* work_counter;
   int32_t* redo;          // short-recurrence kernel: atoms left to the general one, and their count
   int* redo_count;
+  int* late_count;        // those of them that the kernel had worked on
   // method
   int p, q, nu;
   double cg_tol;

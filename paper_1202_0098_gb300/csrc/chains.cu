@@ -1309,7 +1309,10 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
     }
     __syncthreads();
     if (st.bad || st.over) {
-      if (tid == 0) A.redo[atomicAdd(A.redo_count, 1)] = (int32_t)widx;
+      if (tid == 0) {
+        A.redo[atomicAdd(A.redo_count, 1)] = (int32_t)widx;
+        atomicAdd(A.late_count, 1);
+      }
       __syncthreads();
       continue;
     }
@@ -1369,6 +1372,22 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
   }
 }
 
+// counter: see kAtomsCounters.
+__global__ void __launch_bounds__(256) judge_kernel(int* counter, int32_t* redo, const int32_t* order, int64_t n_first,
+                                                    int64_t n_sel, bool mixed) {
+  const int left = counter[1], late = counter[3];
+  __syncthreads();
+  if (chains_pay(mixed, late, n_first - (left - late))) {
+    if (threadIdx.x == 0) counter[0] = (int)n_first;
+    return;
+  }
+  for (int64_t i = n_first + threadIdx.x; i < n_sel; i += 256) redo[left + i - n_first] = order ? order[i] : (int32_t)i;
+  if (threadIdx.x == 0) {
+    counter[0] = (int)n_sel;
+    counter[1] = (int)(left + n_sel - n_first);
+  }
+}
+
 size_t chains_smem_bytes(int clcap, int lnnz_cap, int mcap, size_t elem) {
   const size_t off = (size_t)(clcap + 2 * (mcap / 4) + 1 + lnnz_cap) * sizeof(int);
   return align_up(off, 64) + (size_t)mcap * 4 * (elem == 4 ? 3 * sizeof(float) : 2 * sizeof(double));
@@ -1408,6 +1427,7 @@ mka_status chains_launch_t(const mka_system* sys, const AtomsConfig& cf, const A
   A.slot_bytes = cf.chains_slot;
   A.redo = a.redo;
   A.redo_count = a.counter + 1;
+  A.late_count = a.counter + 3;
   const int grid = (int)std::min<int64_t>(a.n_sel, cf.chains_grid);
   chains_kernel<TV, T, NT><<<(unsigned)grid, NT, cf.chains_smem, st>>>(A);
   count_launches();
@@ -1422,6 +1442,13 @@ mka_status chains_config(const mka_system* sys, int nu, int arith, int ctas_per_
 #define MKA_CFG(TV, T, NT) chains_config_t<TV, T, NT>(nu, ctas_per_sm, cf)
   return MKA_DISPATCH(MKA_CFG, sys->storage, mixed, cf->threads);
 #undef MKA_CFG
+}
+
+mka_status chains_judge(int arith, const AtomsLaunchArgs& a, int64_t n_first, cudaStream_t st) {
+  judge_kernel<<<1, 256, 0, st>>>(a.counter, a.redo, a.order, n_first, a.n_sel, arith != MKA_FP64);
+  count_launches();
+  MKA_CUDA_TRY(cudaGetLastError());
+  return MKA_OK;
 }
 
 mka_status chains_launch(const mka_system* sys, int arith, const AtomsConfig& cf, const AtomsLaunchArgs& a,

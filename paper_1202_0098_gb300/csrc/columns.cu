@@ -1076,7 +1076,7 @@ mka_status config_t(const mka_system* sys, int nu, int max_cl, int max_rows, int
   MKA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, cf.smem));
   if (per_sm < 1) return fail(MKA_ERR_INVALID_ARG, "per-atom working set does not fit in shared memory");
   if (ctas_per_sm > 0) per_sm = std::min(per_sm, ctas_per_sm);
-  cf.per_sm = per_sm;
+  cf.per_sm = cf.general_per_sm = per_sm;
   cf.grid_max = sms * per_sm;
   *out = cf;
   return MKA_OK;
@@ -1164,6 +1164,13 @@ mka_status atoms_launch(const mka_system* sys, int arith, const AtomsConfig& cf,
   if (std::max(a.pick_atoms, a.n_sel) <= cf.single_max && !a.cg_only && !a.mode_b && !a.x0 && !a.prev_s && !a.keep_s && !a.fallback && a.grid <= 0)
     return single_launch(sys, cf, a, st);
   if (cf.chains) {
+    if (a.judge && !a.cg_only && a.n_sel >= 2 * (int64_t)cf.chains_grid) {   // the first wave by itself
+      AtomsLaunchArgs first = a;
+      first.n_sel = cf.chains_grid;
+      mka_status s = chains_launch(sys, arith, cf, first, st);
+      if (!s) s = chains_judge(arith, a, first.n_sel, st);
+      if (s) return s;
+    }
     const mka_status s = chains_launch(sys, arith, cf, a, st);
     if (s || a.cg_only) return s;
   }
@@ -1251,6 +1258,7 @@ mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_para
     a.scratch = scratch;
     a.counter = counter;
     a.redo = counter + kAtomsCounters;
+    a.judge = 1;
     a.red = red;
     s = atoms_launch(sys, prm->arith, cf, a, st);
     if (!s) s = reduced_for(sys, a, st);

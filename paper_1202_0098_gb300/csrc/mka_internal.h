@@ -93,7 +93,8 @@ namespace mka {
 // Configuration of the per-atom kernel for a system, subspace size, arithmetic and CTA size.
 struct AtomsConfig {
   int threads = 256;       // CTA size
-  int per_sm = 0;          // resident CTAs per SM used
+  int per_sm = 0;          // resident CTAs per SM used (of the kernel that runs first)
+  int general_per_sm = 0;  // and of the general kernel
   int grid_max = 0;        // SMs x per_sm
   size_t smem = 0;         // dynamic shared memory per CTA
   size_t slot_bytes = 0;   // global work slot per CTA
@@ -108,7 +109,9 @@ struct AtomsConfig {
 };
 // Subspaces up to this size run the short-recurrence kernel (chains.cu).
 constexpr int kChainsMaxNu = 48;
-// Ints behind AtomsLaunchArgs::counter: queue positions of the two kernels and the count of atoms left over.
+// Ints behind AtomsLaunchArgs::counter: the short recurrences' queue position, the atoms they left over, the general
+// kernel's queue position, and those of the atoms left over that had cost the recurrences' work (the others are seen by
+// their cluster).
 constexpr int kAtomsCounters = 4;
 
 // Arguments of one launch of the per-atom kernel over a selection.
@@ -133,6 +136,7 @@ struct AtomsLaunchArgs {
   char* scratch = nullptr;         // grid x slot_bytes
   int* counter = nullptr;          // [kAtomsCounters], zero in stream order before the launch
   int32_t* redo = nullptr;         // [n_sel] atoms the short-recurrence kernel leaves to the general one
+  int judge = 0;                   // 1: a large selection's first atoms decide whether the rest try the recurrences
   int grid = 0;
   const float* x0 = nullptr;       // learned CG start on the patch [4 n_sel][68], or NULL
   const int32_t* patch = nullptr;  // [n_sel][17]
@@ -196,6 +200,14 @@ mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl,
 mka_status chains_config(const mka_system* sys, int nu, int arith, int ctas_per_sm, AtomsConfig* cf);
 mka_status chains_launch(const mka_system* sys, int arith, const AtomsConfig& cf, const AtomsLaunchArgs& a,
                          cudaStream_t st);
+// Do the short recurrences pay when they leave `late` of n atoms they have worked on to the general kernel? Such an atom
+// costs both kernels; the recurrences take about 0.8 of the general kernel's time in FP64 and half of it in the mixed form. Perfect
+// crystals leave every atom: their Krylov spaces close by symmetry (2,000 atoms, fcc, p = q = 8, FP64: 18 ms
+// without them, 30 with, 21 where the first wave decides; S a hair off the unit matrix likewise).
+__host__ __device__ constexpr bool chains_pay(bool mixed, int64_t late, int64_t n) { return late * (mixed ? 2 : 5) <= n; }
+// Leaves the atoms of a selection from n_first on to the general kernel when the first n_first showed that the
+// recurrences do not pay; else the queue goes on with them.
+mka_status chains_judge(int arith, const AtomsLaunchArgs& a, int64_t n_first, cudaStream_t st);
 // A CTA per column (single.cu; FP64, reading A): sets cf->single_max, and its launch, on the general kernel's slots.
 mka_status single_config(const mka_system* sys, int nu, AtomsConfig* cf);
 mka_status single_launch(const mka_system* sys, const AtomsConfig& cf, const AtomsLaunchArgs& a, cudaStream_t st);

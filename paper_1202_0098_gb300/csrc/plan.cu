@@ -157,6 +157,46 @@ mka_status plan_alloc(mka_plan* P) {
 }
 
 // Enqueue one batch of n atoms (already staged) on the capture stream (recorded into a graph).
+// The short recurrences are tried on up to 64 atoms spread over the system, and dropped for the plan's life when they
+// do not pay (chains_pay): by the system's atoms and not a batch's, so that a sweep's levels do not depend on its batches.
+mka_status plan_trial(mka_plan* P) {
+  const mka_system* sys = P->sys;
+  const int64_t n = std::min<int64_t>(sys->n_atoms, 64), most = std::min(n, P->max_atoms);
+  int64_t late = 0, tried = 0;
+  std::vector<int64_t> sel;
+  for (int64_t off = 0; off < n; off += most) {
+    sel.clear();
+    for (int64_t i = off; i < std::min(n, off + most); ++i) sel.push_back(i * sys->n_atoms / n);
+    MKA_CUDA_TRY(cudaMemcpyAsync(P->res->d_sel, sel.data(), sizeof(int64_t) * sel.size(), cudaMemcpyHostToDevice, P->stream));
+    MKA_CUDA_TRY(cudaMemsetAsync(P->counter, 0, sizeof(int) * kAtomsCounters, P->stream));
+    AtomsLaunchArgs a{};
+    a.sel = P->res->d_sel;
+    a.n_sel = (int64_t)sel.size();
+    a.p = P->prm.p;
+    a.q = P->prm.q;
+    a.cg_tol = P->prm.cg_tol;
+    a.cg_maxit = P->prm.cg_maxit;
+    a.nu_eff = P->res->d_nu_eff;
+    a.cg_iters = P->res->d_cg_iters;
+    a.status = P->res->d_status;
+    a.scratch = P->scratch;
+    a.counter = P->counter;
+    a.redo = P->counter + kAtomsCounters;
+    a.red = P->red;
+    mka_status s = chains_launch(sys, P->prm.arith, P->cf, a, P->stream);
+    if (s) return s;
+    int c[kAtomsCounters] = {};
+    MKA_CUDA_TRY(cudaMemcpyAsync(c, P->counter, sizeof(c), cudaMemcpyDeviceToHost, P->stream));
+    MKA_CUDA_TRY(cudaStreamSynchronize(P->stream));
+    late += c[3];
+    tried += a.n_sel - (c[1] - c[3]);
+  }
+  if (chains_pay(P->prm.arith != MKA_FP64, late, tried)) return MKA_OK;
+  P->cf.chains = 0;
+  P->cf.per_sm = P->cf.general_per_sm;
+  return MKA_OK;
+}
+
 mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   cudaStream_t st = P->capture;
   mka_result* r = P->res;
@@ -313,8 +353,9 @@ mka_status mka_plan_create(mka_system* sys, int64_t max_atoms, const mka_solve_p
     delete P;
     return s;
   }
-  P->grid = (int)std::min<int64_t>(P->max_atoms, P->cf.chains ? P->cf.chains_grid : P->cf.grid_max);
   s = plan_alloc(P);
+  if (!s && P->cf.chains) s = plan_trial(P);
+  P->grid = (int)std::min<int64_t>(P->max_atoms, P->cf.chains ? P->cf.chains_grid : P->cf.grid_max);
   if (s) {
     mka_plan_destroy(P);
     return s;
