@@ -385,7 +385,7 @@ mka_status mka_plan_scalars(mka_plan* plan, double* mu, double* e_band, double* 
 
 /* Device times (ms) of the last batch's two column kernels, from events the
  * graph records around them: the per-atom kernel (cluster, CG, basis,
- * projection) and the batched reduced problems (one lane per column). Either
+ * projection) and the batched reduced problems. Either
  * output may be NULL; waits for that batch's reduced problems to finish. */
 mka_status mka_plan_kernel_ms(mka_plan* plan, float* atoms_ms, float* reduced_ms);
 

@@ -172,8 +172,7 @@ inline size_t kept_buffer_bytes(int64_t n_cols, int nu) {
 inline size_t red_buffer_bytes(int64_t n_cols, int nu) {
   return sizeof(double) * red_block_doubles(nu) * 32 * (size_t)((n_cols + 31) / 32);
 }
-// The batched reduced problems (reduced.cu): one lane per column over the buffer filled by
-// the per-atom kernel; writes eps, w (ranked), the final status and nu_eff, and (cv != NULL)
+// The batched reduced problems (reduced.cu) over the buffer filled by the per-atom kernel; writes eps, w (ranked), the final status and nu_eff, and (cv != NULL)
 // the kept C and V_j of column col0 + c.
 // pick_cols: columns by whose number the form is picked (reduced_rule.cuh).
 mka_status reduced_launch(double* red, int64_t n_cols, int64_t pick_cols, int nu, int32_t* status, int32_t* nu_eff, double* eps,
