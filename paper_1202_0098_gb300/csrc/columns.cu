@@ -55,7 +55,6 @@
 
 #include "atoms.cuh"
 #include "mka_internal.h"
-#include "reduced_rule.cuh"
 
 namespace mka {
 namespace {
@@ -1153,7 +1152,7 @@ mka_status atoms_config(const mka_system* sys, const AtomsShape& sh, int max_cl,
 
 mka_status reduced_for(const mka_system* sys, const AtomsLaunchArgs& a, cudaStream_t st) {
   const int nu = a.p + a.q;
-  return reduced_launch(a.red, 4 * a.n_sel, a.pick_atoms ? system_columns(nu, a.pick_atoms) : 4 * a.n_sel, nu, a.status, a.nu_eff, a.eps, a.w, a.keep ? a.cv : nullptr,
+  return reduced_launch(a.red, 4 * a.n_sel, a.pick_cols ? a.pick_cols : 4 * a.n_sel, nu, a.status, a.nu_eff, a.eps, a.w, a.keep ? a.cv : nullptr,
                         a.col0, st);
 }
 
@@ -1259,6 +1258,10 @@ mka_status launch_columns(mka_system* sys, mka_result* res, const mka_solve_para
     a.counter = counter;
     a.redo = counter + kAtomsCounters;
     a.judge = 1;
+    if (chunk < res->n_sel) {
+      a.pick_atoms = chunk;
+      a.pick_cols = 4 * chunk;
+    }
     a.red = red;
     s = atoms_launch(sys, prm->arith, cf, a, st);
     if (!s) s = reduced_for(sys, a, st);

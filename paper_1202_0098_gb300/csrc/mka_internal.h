@@ -119,9 +119,10 @@ struct AtomsLaunchArgs {
   const int64_t* sel = nullptr;    // device selected atoms
   const int32_t* order = nullptr;  // device work order (selection indices) or NULL
   int64_t n_sel = 0;
-  // Atoms by whose number the kernels are picked (0: n_sel). A sweep's batches pick by the whole system's: the forms round
-  // differently, and an atom's levels may not depend on the batch, nor on the process, that it is in.
-  int64_t pick_atoms = 0;
+  // Atoms, and columns of the reduced problems, by whose number the kernels are picked (0: the selection's). The forms
+  // round differently: a sweep's batches pick by the whole system's, so that an atom's levels do not depend on the batch,
+  // nor on the process, that it is in, and the chunks of one direct solve pick by the full chunk's.
+  int64_t pick_atoms = 0, pick_cols = 0;
   int p = 0, q = 0;
   double cg_tol = 0;
   int cg_maxit = 0;

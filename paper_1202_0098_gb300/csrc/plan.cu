@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "mka_internal.h"
+#include "reduced_rule.cuh"
 
 #ifndef MKA_SOURCE_MARK           // a hash of the sources, given by the build
 #define MKA_SOURCE_MARK "unknown"
@@ -251,7 +252,10 @@ mka_status plan_enqueue(mka_plan* P, int64_t n, const PlanMode& m) {
   a.cv = r->d_cv;
   a.col0 = 0;
   a.mode_b = P->prm.subspace == MKA_SUBSPACE_B;
-  if (m.kind != PLAN_BATCH) a.pick_atoms = P->sys->n_atoms;
+  if (m.kind != PLAN_BATCH) {
+    a.pick_atoms = P->sys->n_atoms;
+    a.pick_cols = system_columns(P->prm.p + P->prm.q, P->sys->n_atoms);
+  }
   MKA_CUDA_TRY(cudaEventRecordWithFlags(P->k0, st, cudaEventRecordExternal));
   mka_status s = atoms_launch(P->sys, P->prm.arith, P->cf, a, st);
   if (s) return s;

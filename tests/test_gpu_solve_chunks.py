@@ -1,0 +1,33 @@
+"""A direct solve that runs in several chunks (the reduced problems' buffer stays within 2 GiB): an atom listed in a full
+chunk and again in the short last one, which by itself would take other kernels, has the same bits in both."""
+import numpy as np
+import pytest
+
+from synth import SK_CARBON_LIKE, lattice_positions
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("arith,storage", [("fp64", "fp64"), ("mixed", "bf16")])
+def test_copies_in_different_chunks(arith, storage):
+    from paper_1202_0098_gb300 import build, mka
+    build.build()
+    p, q = 50, 50
+    per = 8 * (3 * 100 * 100 + 2 * 100) * 4                # bytes of an atom's reduced problems
+    chunk = (2 << 30) // per // 8 * 8
+    pos, box = lattice_positions("diamond", 3.567, 3, 0.08, 0.0, 23)
+    s = mka.mka_build_system(pos, box, SK_CARBON_LIKE, storage, cluster_radius=5.0)
+    try:
+        n = chunk + 5
+        atoms = np.arange(n, dtype=np.int64) % 8
+        res = mka.mka_solve_columns(s, atoms, mka.solve_params(p, q, arith=arith, cg_tol=1e-12 if arith == "fp64" else 1e-7,
+                                                               keep_vectors=False))
+        lv = mka.mka_result_copy_levels(res)
+        mka.mka_result_destroy(res)
+        for k in ("eps", "w", "nu_eff", "status"):
+            x = lv[k].reshape(n, 4, -1)
+            for a in range(8):
+                assert (x[atoms == a] == x[a]).all(), (k, a)
+    finally:
+        mka.mka_system_destroy(s)
