@@ -30,10 +30,10 @@
 // FP32 form by the products' FP32 pipe and shared-memory gathers (a third of the time), then by the latency of the
 // reductions between steps.
 //
-// One thread owns a row of all four columns. In the FP32 form every recurrence runs in FP32 pairs (hi + lo), scalars
-// and dot products included, since rounding at FP32 level would be amplified by the lost orthogonality; S w, z and
-// the Gram matrices take FP32 from the hi parts, as the general kernel does, and H_r comes from the recurrence
-// coefficients. Sums across threads are FP64.
+// One thread owns a row of all four columns. In the FP32 form every recurrence runs in FP32 pairs (hi + lo), scalars,
+// z and dot products included, since rounding at FP32 level would be amplified by the lost orthogonality and at the
+// seam; S w and the Gram matrices take FP32 from the hi parts, as the general kernel does, and H_r comes from the
+// recurrence coefficients. Sums across threads are FP64.
 #include <cuda_bf16.h>
 #include <cuda_pipeline.h>
 #include <cuda_runtime.h>
@@ -413,6 +413,14 @@ __device__ __forceinline__ void row_hs(const TV* __restrict__ valH, const TV* __
   }
 }
 
+// (S x)_row as a pair for a pair x. Out of line: once an atom, and the kernel is sensitive to its own code size.
+template <typename TV>
+__device__ __noinline__ void row_s_pair(const TV* __restrict__ valS, int rb, int e0, int e1, const uint32_t* ent, int i,
+                                        const Vec<float>& x, f2 zero, Pair h[4]) {
+  float sw[4];
+  row_hs<TV>(valS, valS, rb, e0, e1, ent, i, x, zero, h, sw);
+}
+
 // Two values from a T array as a vector load.
 __device__ __forceinline__ void ld2(const float* p, float v[2]) {
   const float2 a = *reinterpret_cast<const float2*>(p);
@@ -622,6 +630,9 @@ __device__ __forceinline__ void check_overlap(ChainState& st, double x) {
 template <typename T, int NT>
 constexpr int chains_min_blocks() { return sizeof(T) == 4 ? 1024 / NT : 768 / NT > 0 ? 768 / NT : 1; }
 
+// Streamed work vectors of a slot.
+__host__ __device__ constexpr int work_vectors(size_t elem) { return elem == 4 ? 11 : 10; }
+
 template <typename TV, typename T, int NT>
 __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(const Args<TV> A) {
   using N = typename Entry<T>::type;
@@ -654,7 +665,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
   T* HW = W + (size_t)nu * m4;
   T* SW = HW + (size_t)nu * m4;
   T* B = SW + (size_t)nu * m4;
-  double* SJd = reinterpret_cast<double*>(slot + align_up(sizeof(T) * ((size_t)3 * nu + 10) * m4, 256));
+  double* SJd = reinterpret_cast<double*>(slot + align_up(sizeof(T) * ((size_t)3 * nu + work_vectors(sizeof(T))) * m4, 256));
   double* tri = SJd + m4;                       // alpha, beta, q.v, z.v of every step, [4][nu][4]
   // shared vectors: X, gathered by the products (CG: p), and the work vector Y (CG: S p). Pairs: X's low half
   // holds s_j during CG; Y's low half (CG: r) is read row by row only and lives in the slot, which lets
@@ -665,7 +676,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
   const Vec<T> SV{B + 2 * m4, B + 3 * m4};      // s_j less its part in the first chain; then a_k
   const Vec<T> BV{B + 4 * m4, B + 5 * m4};      // b_k
   const Vec<T> QV{B + 6 * m4, B + 9 * m4};      // q_{p+1}
-  T* ZV = B + 7 * m4;                           // z
+  const Vec<T> ZV{B + 7 * m4, B + 10 * m4};     // z
   T* SJ = kPair ? X.l : B + 8 * m4;             // CG: s_j
   auto sjrow = [](int r) { return kPair ? xrow<T>(r) : r; };
   T* R = kPair ? Y.l : B;                       // CG: the residual
@@ -1106,9 +1117,9 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
 #pragma unroll
         for (int c = 0; c < 4; ++c) dot_acc(d0[c], h[c], h[c]);
         if (second) {
-          T z[4];
+          N z[4];
           ldv(QV, r, v);
-          ld4(ZV + 4 * r, z);
+          ldv(ZV, r, z);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             dot_acc(d1[c], v[c], h[c]);
@@ -1233,7 +1244,34 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
           }
           __syncthreads();
           if (st.bad) break;
-          // z = sum_n g_n S q_n, and q.v_1, z.v_1
+          // z = S (Q g), and q.v_1, z.v_1. FP64 adds up the g_n S q_n. The second chain's span leans on z, in one of 10^5
+          // columns 300 times as much as in most, and with z from the FP32 S q_n rho of such columns was off by up to 9e-7
+          // (most: 1e-8); so the pair form multiplies the pair Q g by S once more, with compensated sums, and keeps z as a
+          // pair: 1.6e-7 at most over 4e5 atoms of three systems, for 2 % of the kernel's time.
+          if constexpr (kPair) {
+            const Vec<T> QG{ZV.h, Y.l};
+            for (int r = tid; r < m; r += NT) {
+              N y[4];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) set_zero(y[c]);
+              for (int k = 0; k < A.p; ++k) {
+                T q[4];
+                ld4(W + (size_t)k * m4 + 4 * r, q);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) dot_acc(y[c], q[c], gv[c * A.p + k]);
+              }
+#pragma unroll
+              for (int c = 0; c < 4; ++c) y[c] = renorm(y[c].h, y[c].l);
+              stv(QG, r, y);
+            }
+            __syncthreads();                     // gv, within X, has been read
+            for (int r = tid; r < m; r += NT) {
+              N y[4];
+              ldv(QG, r, y);
+              stv(X, xrow<T>(r), y);
+            }
+            __syncthreads();
+          }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             set_zero(d0[c]);
@@ -1242,25 +1280,27 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
           for (int r = tid; r < m; r += NT) {
             N v[4];
             ldv(PV, r, v);
-            N zs[4];
+            N z[4];
+            if constexpr (kPair) {
+              row_s_pair<TV>(A.valS, rbase[r >> 2], lrow[r >> 2], lrow[(r >> 2) + 1], ent, r & 3, X, A.zero, z);
+            } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) set_zero(zs[c]);
-            for (int k = 0; k < A.p; ++k) {
-              T s[4];
-              ld4(SW + (size_t)k * m4 + 4 * r, s);
+              for (int c = 0; c < 4; ++c) set_zero(z[c]);
+              for (int k = 0; k < A.p; ++k) {
+                T s[4];
+                ld4(SW + (size_t)k * m4 + 4 * r, s);
 #pragma unroll
-              for (int c = 0; c < 4; ++c) dot_acc(zs[c], s[c], gv[c * A.p + k]);
+                for (int c = 0; c < 4; ++c) dot_acc(z[c], s[c], gv[c * A.p + k]);
+              }
             }
             N q[4];
-            T z[4];
             ldv(QV, r, q);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-              z[c] = (T)to_double(zs[c]);
               dot_acc(d0[c], q[c], v[c]);
               dot_acc(d1[c], z[c], v[c]);
             }
-            st4(ZV + 4 * r, z[0], z[1], z[2], z[3]);
+            stv(ZV, r, z);
           }
           warp_partial(d0, red, 0, 2);
           warp_partial(d1, red, 1, 2);
@@ -1394,7 +1434,7 @@ size_t chains_smem_bytes(int clcap, int lnnz_cap, int mcap, size_t elem) {
 }
 
 size_t chains_slot_bytes(int nu, int mcap, size_t elem) {
-  return align_up(elem * ((size_t)3 * nu + 10) * mcap * 4, 256) +
+  return align_up(elem * ((size_t)3 * nu + work_vectors(elem)) * mcap * 4, 256) +
          align_up(sizeof(double) * (4 * (size_t)mcap + 16 * (size_t)nu), 256);
 }
 
