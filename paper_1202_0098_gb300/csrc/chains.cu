@@ -413,14 +413,6 @@ __device__ __forceinline__ void row_hs(const TV* __restrict__ valH, const TV* __
   }
 }
 
-// (S x)_row as a pair for a pair x. Out of line: once an atom, and the kernel is sensitive to its own code size.
-template <typename TV>
-__device__ __noinline__ void row_s_pair(const TV* __restrict__ valS, int rb, int e0, int e1, const uint32_t* ent, int i,
-                                        const Vec<float>& x, f2 zero, Pair h[4]) {
-  float sw[4];
-  row_hs<TV>(valS, valS, rb, e0, e1, ent, i, x, zero, h, sw);
-}
-
 // Two values from a T array as a vector load.
 __device__ __forceinline__ void ld2(const float* p, float v[2]) {
   const float2 a = *reinterpret_cast<const float2*>(p);
@@ -593,6 +585,42 @@ __device__ __noinline__ void gram_s(const float* W, const float* SW, int m, int 
         R[(size_t)(nu * nu + b * nu + a) * 32] = v;
         if (Gs) Gs[c * gs_stride + b * (b + 1) / 2 + a] = v;
       }
+  }
+}
+
+// z = S (Q g) of the pair form into ZV, by way of X (free at the seam; gv lies within it) and `spare`. Out of line, as
+// gram and gram_s: once an atom, and the kernel is sensitive to its own code size.
+template <typename TV>
+__device__ __noinline__ void seam_z(const TV* __restrict__ valS, f2 zero, const float* W, int p, int m, int m4, const Pair* gv,
+                                    const Vec<float>& X, float* spare, const Vec<float>& ZV, const int* rbase, const int* lrow,
+                                    const uint32_t* ent) {
+  const Vec<float> QG{ZV.h, spare};
+  for (int r = threadIdx.x; r < m; r += blockDim.x) {
+    Pair y[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) set_zero(y[c]);
+    for (int k = 0; k < p; ++k) {
+      float q[4];
+      ld4(W + (size_t)k * m4 + 4 * r, q);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) dot_acc(y[c], q[c], gv[c * p + k]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) y[c] = renorm(y[c].h, y[c].l);
+    stv(QG, r, y);
+  }
+  __syncthreads();                     // gv has been read
+  for (int r = threadIdx.x; r < m; r += blockDim.x) {
+    Pair y[4];
+    ldv(QG, r, y);
+    stv(X, xrow<float>(r), y);
+  }
+  __syncthreads();
+  for (int r = threadIdx.x; r < m; r += blockDim.x) {
+    Pair z[4];
+    float sw[4];
+    row_hs<TV>(valS, valS, rbase[r >> 2], lrow[r >> 2], lrow[(r >> 2) + 1], ent, r & 3, X, zero, z, sw);
+    stv(ZV, r, z);
   }
 }
 
@@ -1247,31 +1275,8 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
           // z = S (Q g), and q.v_1, z.v_1. FP64 adds up the g_n S q_n. The second chain's span leans on z, in one of 10^5
           // columns 300 times as much as in most, and with z from the FP32 S q_n rho of such columns was off by up to 9e-7
           // (most: 1e-8); so the pair form multiplies the pair Q g by S once more, with compensated sums, and keeps z as a
-          // pair: 1.6e-7 at most over 4e5 atoms of three systems, for 2 % of the kernel's time.
-          if constexpr (kPair) {
-            const Vec<T> QG{ZV.h, Y.l};
-            for (int r = tid; r < m; r += NT) {
-              N y[4];
-#pragma unroll
-              for (int c = 0; c < 4; ++c) set_zero(y[c]);
-              for (int k = 0; k < A.p; ++k) {
-                T q[4];
-                ld4(W + (size_t)k * m4 + 4 * r, q);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) dot_acc(y[c], q[c], gv[c * A.p + k]);
-              }
-#pragma unroll
-              for (int c = 0; c < 4; ++c) y[c] = renorm(y[c].h, y[c].l);
-              stv(QG, r, y);
-            }
-            __syncthreads();                     // gv, within X, has been read
-            for (int r = tid; r < m; r += NT) {
-              N y[4];
-              ldv(QG, r, y);
-              stv(X, xrow<T>(r), y);
-            }
-            __syncthreads();
-          }
+          // pair: 1.6e-7 at most over 4.5e5 atoms of three systems, for 2 % of the kernel's time.
+          if constexpr (kPair) seam_z<TV>(A.valS, A.zero, W, A.p, m, m4, gv, X, Y.l, ZV, rbase, lrow, ent);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             set_zero(d0[c]);
@@ -1282,7 +1287,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
             ldv(PV, r, v);
             N z[4];
             if constexpr (kPair) {
-              row_s_pair<TV>(A.valS, rbase[r >> 2], lrow[r >> 2], lrow[(r >> 2) + 1], ent, r & 3, X, A.zero, z);
+              ldv(ZV, r, z);
             } else {
 #pragma unroll
               for (int c = 0; c < 4; ++c) set_zero(z[c]);
@@ -1300,7 +1305,7 @@ __global__ void __launch_bounds__(NT, chains_min_blocks<T, NT>()) chains_kernel(
               dot_acc(d0[c], q[c], v[c]);
               dot_acc(d1[c], z[c], v[c]);
             }
-            stv(ZV, r, z);
+            if constexpr (!kPair) stv(ZV, r, z);
           }
           warp_partial(d0, red, 0, 2);
           warp_partial(d1, red, 1, 2);
