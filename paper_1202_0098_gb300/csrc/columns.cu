@@ -1348,6 +1348,7 @@ mka_status run_columns_static(const mka_system* sys, const int64_t* h_atoms, int
     a.status = status + 4 * off;
     a.keep = 0;
     a.grid = (int)std::min<int64_t>(std::min<int64_t>(cnt, slots_fit), cf.grid_max);
+    if (chunk < n_sel) a.pick_cols = 4 * chunk;
     // The counter must start at zero; the chunk's atom list is copied in; slots and the reduced
     // buffer need no clearing (every entry is written before it is read).
     MKA_CUDA_TRY(cudaMemsetAsync(base, 0, 256, st));
